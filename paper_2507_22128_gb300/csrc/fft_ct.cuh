@@ -116,7 +116,6 @@ __device__ __forceinline__ void pass_ct(const cplx<R>* __restrict__ src, cplx<R>
   constexpr int TOTAL = B * IPR;
   constexpr int NIT = (TOTAL + kFftThreads - 1) / kFftThreads;
   constexpr int STRIDE = padded_len(L);
-  constexpr int TWSHIFT = kTwLog - (LOGP + LR);
   // padi(x + r c) == padi(x) + r (c + c / 16) when c is a multiple of 16
   constexpr bool kLinIn = (IPR % 16) == 0;
   // outputs o + r P: linear when P is a multiple of 16, or when all RAD of
@@ -151,7 +150,7 @@ __device__ __forceinline__ void pass_ct(const cplx<R>* __restrict__ src, cplx<R>
         if (!kZin || ct_outer<RAD>(r)) v[r] = rs[padi(i + r * IPR)];
     }
     if constexpr (LOGP > 0) {
-      if (k) apply_twiddles<R, DIR, RAD>(v, tw, k, TWSHIFT);
+      if (k) apply_twiddles<R, DIR, RAD>(v, tw, k, LOGP + LR);
     }
     if constexpr (kZin) dft_zin<RAD, DIR>(v);
     else dft<RAD, DIR>(v);

@@ -837,7 +837,7 @@ int image_to_planes(Job* job, Part& pt, const R* image, cudaStream_t st) {
 template <typename R>
 int planes_to_image(Job* job, Part& pt, R* image, cudaStream_t st) {
   const XformGeom g = plane_geom(job, pt, false);
-  RIX_TRY(inv_cols<R>(job->ctx, g, pt.resid_planes.as<cplx<R>>(), kOpNone, nullptr, nullptr,
+  RIX_TRY(inv_cols<R>(job->ctx, g, pt.resid_planes.as<cplx<R>>(), kOpNone, nullptr,
                       pt.tbuf.as<cplx<R>>(), st));
   const double sc = pt.wsum > 0.0 ? 1.0 / pt.wsum : 0.0;
   const int G = inv_rows_groups<R>(job->ctx, g, 16);
@@ -1014,7 +1014,7 @@ int op_psf_tiled(Job* job, int p, cudaStream_t st) {
     a.out = pt.resid_planes.p;
     a.vis_in = vis;
     if ((rc = launch_tiles<R, kGrid>(job, a, st)) != RIX_OK) break;
-    if ((rc = inv_cols<R>(job->ctx, g, pt.resid_planes.as<cplx<R>>(), kOpNone, nullptr, nullptr,
+    if ((rc = inv_cols<R>(job->ctx, g, pt.resid_planes.as<cplx<R>>(), kOpNone, nullptr,
                           pt.tbuf.as<cplx<R>>(), st)) != RIX_OK)
       break;
     if ((rc = inv_rows<R>(job->ctx, g, pt.tbuf.as<cplx<R>>(), tile, sc, 0, st, pt.groups.as<R>(), G)) != RIX_OK) break;
@@ -1101,7 +1101,7 @@ int op_psf(Job* job, int p, cudaStream_t st) {
       if ((rc = launch_tiles<R, kPsf>(job, a, st)) != RIX_OK) break;
     }
     const XformGeom g = plane_geom(job, pt, true);
-    if ((rc = inv_cols<R>(job->ctx, g, pp, kOpNone, nullptr, nullptr, tt, st)) != RIX_OK) break;
+    if ((rc = inv_cols<R>(job->ctx, g, pp, kOpNone, nullptr, tt, st)) != RIX_OK) break;
     const double sc = pt.wsum > 0.0 ? 1.0 / pt.wsum : 0.0;
     if ((rc = inv_rows<R>(job->ctx, g, tt, pt.psf.as<R>(), sc, 0, st)) != RIX_OK) break;
     // centred spectrum of the 2N x 2N PSF on the 2N grid
@@ -1145,7 +1145,7 @@ int op_grid_into_scratch(Job* job, int p, const float2* vis, float* image_out, f
   a.vis_in = vis;
   RIX_TRY(launch_tiles<float, kGrid>(job, a, st));
   const XformGeom g = plane_geom(job, pt, false);
-  RIX_TRY(inv_cols<float>(job->ctx, g, planes, kOpNone, nullptr, nullptr, tbuf, st));
+  RIX_TRY(inv_cols<float>(job->ctx, g, planes, kOpNone, nullptr, tbuf, st));
   const double sc = pt.wsum > 0.0 ? 1.0 / pt.wsum : 0.0;
   return inv_rows<float>(job->ctx, g, tbuf, image_out, sc, 0, st, group_imgs, std::max(max_groups, 1));
 }

@@ -39,7 +39,7 @@ template <typename R>
 int spec_to_img(Job* job, Part& pt, const cplx<R>* spec, int op, const void* tab, R* out, double scale,
                 int accumulate, cudaStream_t st) {
   const XformGeom g = fill_geom(job->desc.n);
-  RIX_TRY(inv_cols<R>(job->ctx, g, spec, op, tab, nullptr, pt.ft_a.as<cplx<R>>(), st));
+  RIX_TRY(inv_cols<R>(job->ctx, g, spec, op, tab, pt.ft_a.as<cplx<R>>(), st));
   return inv_rows<R>(job->ctx, g, pt.ft_a.as<cplx<R>>(), out, scale, accumulate, st);
 }
 
@@ -50,13 +50,13 @@ int spec_to_img(Job* job, Part& pt, const cplx<R>* spec, int op, const void* tab
 // spectrum are formed and transformed; the inverse row pass completes the
 // others by conjugation.
 template <typename R>
-int convolve(Job* job, Part& pt, const R* x, int op, const void* tab, const void* tab2, R* out, double scale,
+int convolve(Job* job, Part& pt, const R* x, int op, const void* tab, R* out, double scale,
              int accumulate, cudaStream_t st) {
   XformGeom g = fill_geom(job->desc.n);
   g.S = job->desc.n + 1;
   g.herm = 1;
   RIX_TRY(fwd_rows<R>(job->ctx, g, x, pt.ft_a.as<cplx<R>>(), st));
-  RIX_TRY(conv_cols<R>(job->ctx, g, pt.ft_a.as<cplx<R>>(), op, tab, tab2, pt.ft_b.as<cplx<R>>(), st));
+  RIX_TRY(conv_cols<R>(job->ctx, g, pt.ft_a.as<cplx<R>>(), op, tab, pt.ft_b.as<cplx<R>>(), st));
   return inv_rows<R>(job->ctx, g, pt.ft_b.as<cplx<R>>(), out, scale, accumulate, st);
 }
 
@@ -495,7 +495,7 @@ int phi_from_coef(Job* job, int p, const cplx<R>* coef, cplx<R>* spec, cplx<R>* 
                                                                        pt.ring_count, n, spec);
   RIX_LAUNCH_CHECK();
   const XformGeom g = fill_geom(n);
-  RIX_TRY(inv_cols<R>(job->ctx, g, spec, kOpNone, nullptr, nullptr, T, st));
+  RIX_TRY(inv_cols<R>(job->ctx, g, spec, kOpNone, nullptr, T, st));
   return inv_rows<R>(job->ctx, g, T, out, scale, accumulate, st);
 }
 
@@ -572,7 +572,7 @@ int publish(Job* job, int p, int cycle, cudaStream_t st) {
                                                                        pt.outbox[cycle & 1].as<cplx<R>>());
     RIX_LAUNCH_CHECK();
   } else {
-    RIX_TRY(convolve<R>(job, pt, ibar, kOpMulReal, gam + p * tot, nullptr, pt.outbox[cycle & 1].as<R>(), inv, 0, st));
+    RIX_TRY(convolve<R>(job, pt, ibar, kOpMulReal, gam + p * tot, pt.outbox[cycle & 1].as<R>(), inv, 0, st));
     if (job->n_part == 2) {
       // Gamma_q = 1 - Gamma_p and crop F^-1 F pad = identity, so
       // Gamma_q i_bar = i_bar - Phi_p: rho_{q->p} += Phi_p - i_bar
@@ -585,7 +585,7 @@ int publish(Job* job, int p, int cycle, cudaStream_t st) {
     }
   }
   for (int q = 0; q < job->n_part; ++q)
-    if (q != p) RIX_TRY(convolve<R>(job, pt, ibar, kOpMulReal, gam + q * tot, nullptr, pt.rho[q].as<R>(), -inv, 1, st));
+    if (q != p) RIX_TRY(convolve<R>(job, pt, ibar, kOpMulReal, gam + q * tot, pt.rho[q].as<R>(), -inv, 1, st));
   return RIX_OK;
 }
 
@@ -766,7 +766,7 @@ int op_msclean(Job* job, int p, const rix_msclean_params* prm, R* delta_out, cud
     for (int t = s; t < ns && rc == RIX_OK; ++t) {
       R* pst = pt.ms_P.as<R>() + (int64_t)(s * ns + t) * tot;
       ::rix::note_launch(); k_cmul3<R><<<blocks_for(ctx, tot), 256, 0, st>>>(bspec + s * tot, bspec + t * tot, pspec, dspec, tot);
-      if ((rc = inv_cols<R>(ctx, g2, dspec, kOpNone, nullptr, nullptr, t2, st)) != RIX_OK) break;
+      if ((rc = inv_cols<R>(ctx, g2, dspec, kOpNone, nullptr, t2, st)) != RIX_OK) break;
       if ((rc = inv_rows<R>(ctx, g2, t2, pst, inv, 0, st)) != RIX_OK) break;
       if (t != s && cudaMemcpyAsync(pt.ms_P.as<R>() + (int64_t)(t * ns + s) * tot, pst, tot * sizeof(R),
                                     cudaMemcpyDeviceToDevice, st) != cudaSuccess)

@@ -165,14 +165,14 @@ struct Ctx {
   int jobs = 0;
   int num_sms = 0;
   cudaStream_t mem_stream = nullptr;   // stream-ordered allocation and release
-  DevBuf tw32, tw64;          // FFT twiddle tables, length kTwMax
+  DevBuf tw32, tw64;          // FFT twiddle tables, 2 kTwMax entries (fft_init_twiddles)
 };
 
 constexpr int kTwLog = 14;
 constexpr int kTwMax = 1 << kTwLog;   // largest 1D FFT length (4N for N = 4096)
 
 // ---------------------------------------------------------------------------
-// FFT plans (see k_fft.cu)
+// transforms (see k_fft.cu)
 // ---------------------------------------------------------------------------
 enum FactorMode : int {
   kFacNone = 0,     // value * (-1)^(a+b)
@@ -189,7 +189,7 @@ struct XformGeom {
   const void* corr;            // Real [M][M] or null
   const double* nm1;           // double [M][M]: n - 1 per pixel (kFacPhase)
   double w0, dw;               // plane p sits at w0 + p * dw (kFacPhase)
-  int herm = 0;                // inverse rows: complete columns [S, L) by conjugate symmetry
+  int herm = 0;                // inverse rows: complete columns [S, L) by conjugate symmetry (lo = 0)
   // kFacPhase, optional: cplx [nplanes][M][M] of corr * exp(-2 pi i w_p (n-1)),
   // the factors tabulated once per job (build_screen_table); corr and nm1
   // are then not read by the row passes
@@ -209,14 +209,15 @@ template <typename R>
 int fwd_rows(const Ctx* ctx, const XformGeom& g, const R* img, cplx<R>* T, cudaStream_t st);
 template <typename R>
 int fwd_cols(const Ctx* ctx, const XformGeom& g, const cplx<R>* T, cplx<R>* spec, cudaStream_t st);
-// spectral operator applied between the forward and inverse column transforms
-enum SpecOp : int { kOpNone = 0, kOpMulReal = 1, kOpMulCplx = 2, kOpAxpyReal = 3 };
+// spectral operator (times the real or complex table tab) applied on the way
+// into the inverse transform, or between conv_cols' two transforms
+enum SpecOp : int { kOpNone = 0, kOpMulReal = 1, kOpMulCplx = 2 };
 template <typename R>
-int inv_cols(const Ctx* ctx, const XformGeom& g, const cplx<R>* spec, int op, const void* tab,
-             const void* tab2, cplx<R>* T, cudaStream_t st);
+int inv_cols(const Ctx* ctx, const XformGeom& g, const cplx<R>* spec, int op, const void* tab, cplx<R>* T,
+             cudaStream_t st);
 template <typename R>
-int conv_cols(const Ctx* ctx, const XformGeom& g, const cplx<R>* Tin, int op, const void* tab,
-              const void* tab2, cplx<R>* Tout, cudaStream_t st);
+int conv_cols(const Ctx* ctx, const XformGeom& g, const cplx<R>* Tin, int op, const void* tab, cplx<R>* Tout,
+              cudaStream_t st);
 // Inverse row pass: img = (accumulate ? img : 0) + scale * the planes' sum.
 // With several planes it may split them into G groups (inv_rows_groups, at
 // most max_groups; -1 = the pass's own limit), each summed into an image of
@@ -228,6 +229,10 @@ int inv_rows(const Ctx* ctx, const XformGeom& g, const cplx<R>* T, R* img, doubl
 // the number of plane groups inv_rows uses for g with at most max_groups
 template <typename R>
 int inv_rows_groups(const Ctx* ctx, const XformGeom& g, int max_groups);
+
+// img = (accumulate ? img : 0) + the sum of G images of n values (k_fft.cu)
+template <typename R>
+int sum_groups(const Ctx* ctx, R* img, const R* parts, int G, int64_t n, int accumulate, cudaStream_t st);
 
 int fft_init_twiddles(Ctx* ctx);
 
@@ -474,7 +479,7 @@ struct FistaLoop {
   const cplx<R>* c;
   R* d;                    // N x N: 2 crop F^-1 c, formed by the loop
   const R* state;          // [max Mx, max |residual| of cycle 1]
-  const cplx<R>* tw;       // twiddle table, length kTwMax
+  const cplx<R>* tw;       // twiddle table (fft_init_twiddles)
   unsigned int* barrier;   // arrival counter (zeroed by the call, stream-ordered)
   int* status;             // the job's status word
   double lambda, lambda_rel;
