@@ -3,13 +3,14 @@
 //
 // The arrival counter only grows during a launch: barrier k completes when it
 // reaches (k + 1) * gridDim.x.  The host zeroes it, stream-ordered, before each
-// launch.  Arrival is a release add at GPU scope after a CTA barrier and a
-// fence; the wait is an acquire load at GPU scope followed by a fence and a
-// CTA barrier, so every write of every CTA before the barrier is visible to
-// every thread after it.
+// launch.  Arrival is a release add at GPU scope after a CTA barrier (which
+// the release is cumulative over); the wait is an acquire load at GPU scope
+// followed by a CTA barrier, so every write of every CTA before the barrier is
+// visible to every thread after it.
 //
-// The wait ends after kBarrierTimeoutNs of global time or kBarrierMaxSpins
-// polls, whichever comes first.  The CTA that gives up stores RIX_ETIMEOUT in
+// The wait ends after kBarrierTimeoutNs of global time (counted from its 64th
+// poll) or kBarrierMaxSpins polls, whichever comes first.  The first polls
+// follow one another without a sleep: most waits end within them.  The CTA that gives up stores RIX_ETIMEOUT in
 // the job's status word and the barrier returns false; a CTA that sees a
 // non-zero status while waiting gives up at once.  Callers return on false.
 #pragma once
@@ -45,29 +46,33 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
+// polls *p until it reaches `target` (bounded, see above); false when the wait
+// gave up.  One thread per CTA.
+__device__ __forceinline__ bool poll_counter(const unsigned int* p, unsigned int target, int* status) {
+  unsigned int spins = 0;
+  unsigned long long t0 = 0;
+  while (ld_acquire_gpu(p) < target) {
+    if ((++spins & 63u) == 0) {
+      if (*reinterpret_cast<volatile int*>(status) != 0) return false;
+      const unsigned long long t = global_ns();
+      if (t0 == 0) t0 = t;
+      if (spins >= kBarrierMaxSpins || t - t0 > kBarrierTimeoutNs) {
+        atomicCAS(status, 0, RIX_ETIMEOUT);
+        return false;
+      }
+    }
+    if (spins > 16) __nanosleep(32);
+  }
+  return true;
+}
+
 __device__ __forceinline__ bool grid_barrier(GridBarrier& b) {
   __shared__ int ok;
   __syncthreads();
   b.target += gridDim.x;
   if (threadIdx.x == 0) {
-    int good = 1;
-    __threadfence();
     red_release_gpu_add(b.count, 1u);
-    const unsigned long long t0 = global_ns();
-    unsigned int spins = 0;
-    while (ld_acquire_gpu(b.count) < b.target) {
-      if ((++spins & 63u) == 0) {
-        if (*reinterpret_cast<volatile int*>(b.status) != 0) { good = 0; break; }
-        if (spins >= kBarrierMaxSpins || global_ns() - t0 > kBarrierTimeoutNs) {
-          atomicCAS(b.status, 0, RIX_ETIMEOUT);
-          good = 0;
-          break;
-        }
-      }
-      __nanosleep(32);
-    }
-    __threadfence();
-    ok = good;
+    ok = poll_counter(b.count, b.target, b.status);
   }
   __syncthreads();
   return ok != 0;

@@ -256,28 +256,36 @@ __device__ __forceinline__ void rows_fwd_syn_unit(const R* __restrict__ ll, cons
     }
   }
   __syncthreads();
-  // rows, computed by the transform's first pass as it loads them: complex
-  // row q = x[b0 + 2q] + i x[b0 + 2q + 1], centred as in rows_fwd_unit
-  // (position p holds column (p + N/2) mod L; the pruned half is zero)
-  auto ld_x = [&](int q, int p) -> C {
-    const int c = (p + H) & (L - 1);
-    const int kc = c >> 1;
-    const bool oc = c & 1;
-    const R* t0a = tv + (2 * q) * H;                  // cx = 0, row 2q
-    const R* t1a = tv + (2 * B + 2 * q) * H;          // cx = 1, row 2q
-    R va = R(0), vb = R(0);
+  // rows: complex row q = x[b0 + 2q] + i x[b0 + 2q + 1], centred as in
+  // rows_fwd_unit (column c at position (c - N/2) mod L).  A thread forms two
+  // adjacent columns of the pair of rows from the five coefficients per
+  // subband and row that they share.
+  for (int e = threadIdx.x; e < B * H; e += kFftThreads) {
+    const int q = e / H, kc = e - (e / H) * H;        // columns 2 kc and 2 kc + 1
+    const R* t0 = tv + (2 * q) * H;                   // cx = 0, row 2q (row 2q + 1 after it)
+    const R* t1 = tv + (2 * B + 2 * q) * H;           // cx = 1
+    R a0[4], a1[4], c0[4], c1[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int kk = (kc - j) & (H - 1);
-      const R lo = oc ? tp.lo(2 * j + 1) : tp.lo(2 * j);
-      const R hi = oc ? tp.hi(2 * j + 1) : tp.hi(2 * j);
-      va += lo * t0a[kk] + hi * t1a[kk];
-      vb += lo * t0a[H + kk] + hi * t1a[H + kk];
+      a0[j] = t0[kk]; c0[j] = t0[H + kk];
+      a1[j] = t1[kk]; c1[j] = t1[H + kk];
     }
-    const bool odd = (c + b0) & 1;
-    return cpx<C>(odd ? -va : va, odd ? vb : -vb);
-  };
-  const C* res = fft_ct<R, -1, LOGL, B, true, false>(s, s2, tw, ld_x);
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+      R va = R(0), vb = R(0);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        va += tp.lo(2 * j + o) * a0[j] + tp.hi(2 * j + o) * a1[j];
+        vb += tp.lo(2 * j + o) * c0[j] + tp.hi(2 * j + o) * c1[j];
+      }
+      const int c = 2 * kc + o;
+      const bool odd = (c + b0) & 1;
+      s[q * STRIDE + padi((c - H) & (L - 1))] = cpx<C>(odd ? -va : va, odd ? vb : -vb);
+    }
+  }
+  __syncthreads();
+  const C* res = fft_ct<R, -1, LOGL, B, true, false>(s, s2, tw);
   constexpr int NO = B * F::S;
   for (int e = threadIdx.x; e < NO; e += kFftThreads) {
     const int q = e % B, j = e / B;
@@ -666,34 +674,14 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 && LOGL <= 12 ? 2 
 // completed units of a stage: release after the CTA's writes
 __device__ __forceinline__ void flow_done(unsigned int* ctr) {
   __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    red_release_gpu_add(ctr, 1u);
-  }
+  if (threadIdx.x == 0) red_release_gpu_add(ctr, 1u);
 }
 
 // wait until *ctr reaches `target`, then acquire (every thread of the CTA
 // sees the stage's writes); false when the wait gave up
 __device__ __forceinline__ bool flow_wait(const unsigned int* ctr, unsigned int target, int* status) {
   __shared__ int ok;
-  if (threadIdx.x == 0) {
-    int good = 1;
-    const unsigned long long t0 = global_ns();
-    unsigned int spins = 0;
-    while (ld_acquire_gpu(ctr) < target) {
-      if ((++spins & 63u) == 0) {
-        if (*reinterpret_cast<volatile int*>(status) != 0) { good = 0; break; }
-        if (spins >= kBarrierMaxSpins || global_ns() - t0 > kBarrierTimeoutNs) {
-          atomicCAS(status, 0, RIX_ETIMEOUT);
-          good = 0;
-          break;
-        }
-      }
-      __nanosleep(32);
-    }
-    __threadfence();
-    ok = good;
-  }
+  if (threadIdx.x == 0) ok = poll_counter(ctr, target, status);
   __syncthreads();
   return ok != 0;
 }

@@ -128,31 +128,57 @@ __device__ __forceinline__ void dwt_tile(const R* __restrict__ src, int lds, int
   }
   cp_async_wait_all();
   __syncthreads();
-  for (int t = threadIdx.x; t < TIN * TB; t += blockDim.x) {
-    const int r = t / TB, xx = t - r * TB;
-    R a = R(0), d = R(0);
+  // rows: a thread forms four adjacent outputs of one row from the 2 * 4 + K - 2
+  // inputs they share (a load per tap and output otherwise: shared-memory
+  // loads, not FMAs, bound the tile); threads along the rows, whose odd stride
+  // keeps them on different banks
+  constexpr int XG = 4;
+  for (int t = threadIdx.x; t < TIN * (TB / XG); t += blockDim.x) {
+    const int r = t % TIN, xx = (t / TIN) * XG;
+    R w[2 * XG + K - 2];
 #pragma unroll
-    for (int i = 0; i < K; ++i) {
-      const R w = tin[r][2 * xx + i];
-      a += tp.lo(i) * w;
-      d += tp.hi(i) * w;
+    for (int i = 0; i < 2 * XG + K - 2; ++i) w[i] = tin[r][2 * xx + i];
+#pragma unroll
+    for (int u = 0; u < XG; ++u) {
+      R a = R(0), d = R(0);
+#pragma unroll
+      for (int i = 0; i < K; ++i) {
+        a += tp.lo(i) * w[2 * u + i];
+        d += tp.hi(i) * w[2 * u + i];
+      }
+      trow[r][xx + u] = a;
+      trow[r][TB + xx + u] = d;
     }
-    trow[r][xx] = a;
-    trow[r][TB + xx] = d;
   }
   __syncthreads();
+  // columns: a thread forms YG adjacent outputs, low and high, of one of the
+  // 2 TB columns, a window of K rows sliding down it
+  constexpr int YG = 2 * TB * TB / 256;
+  const int col = threadIdx.x % (2 * TB), ty0 = (threadIdx.x / (2 * TB)) * YG;
+  const int cx = col / TB, tx = col - cx * TB;
+  const int x = x0 + tx;
+  R w[K];
 #pragma unroll
-  for (int k = 0; k < TB * TB / 256; ++k) {
-    const int pidx = threadIdx.x + 256 * k;
-    const int ty = pidx / TB, tx = pidx - ty * TB;
-    const int y = y0 + ty, x = x0 + tx;
+  for (int i = 2; i < K; ++i) w[i] = trow[2 * ty0 + i - 2][col];
+#pragma unroll
+  for (int u = 0; u < YG; ++u) {
+    const int ty = ty0 + u, y = y0 + ty;
+#pragma unroll
+    for (int i = 0; i < K - 2; ++i) w[i] = w[i + 2];
+    w[K - 2] = trow[2 * ty + K - 2][col];
+    w[K - 1] = trow[2 * ty + K - 1][col];
+    R gl = R(0), gh = R(0);
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      gl += tp.lo(i) * w[i];
+      gh += tp.hi(i) * w[i];
+    }
     if (y < h && x < h) {
+      const int pidx = ty * TB + tx;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int cy = q >> 1, cx = q & 1;
-        R g = R(0);
-#pragma unroll
-        for (int i = 0; i < K; ++i) g += (cy ? tp.hi(i) : tp.lo(i)) * trow[2 * ty + i][cx * TB + tx];
+      for (int cy = 0; cy < 2; ++cy) {
+        const R g = cy ? gh : gl;
+        const int q = 2 * cy + cx;
         const int64_t idx = (int64_t)(cy * h + y) * ld + cx * h + x;
         if (q == 0 && !last) {
           ll[(int64_t)y * ld + x] = g;
@@ -219,37 +245,58 @@ __device__ __forceinline__ void idwt_tile(const R* __restrict__ llin, const R* _
     }
   }
   __syncthreads();
-  // rows: tr[cy][rk][c] = sum over the K/2 taps of the parity of c
-  for (int t = threadIdx.x; t < 2 * RK * kTS; t += blockDim.x) {
-    const int cy = t / (RK * kTS), rem = t - cy * RK * kTS;
-    const int rk = rem / kTS, cl = rem - rk * kTS;
-    const int c = c0 + cl;
-    const bool odd = c & 1;
-    const int kc = (c >> 1) - kb_c;             // tap i = 2 j + (c & 1) reads coefficient (c - i) / 2
-    R v2 = R(0);
+  // rows: tr[cy][rk][c] = sum over the K/2 taps of the parity of c; tap
+  // i = 2 j + (c & 1) reads coefficient (c - i) / 2.  A thread forms four
+  // adjacent c (two of each parity) from the K/2 + 1 coefficients they share
+  // in each of the two subbands (c0 and m0 are even).
+  constexpr int HK = K / 2;
+  for (int t = threadIdx.x; t < 2 * RK * (kTS / 4); t += blockDim.x) {
+    const int rk = t % RK, rem = t / RK;
+    const int cy = rem & 1, cl = (rem >> 1) * 4;
+    R q0[HK + 1], q1[HK + 1];                    // coefficients kc + 1 - i
+    const int kc = (cl >> 1) + HK;
 #pragma unroll
-    for (int j = 0; j < K / 2; ++j) {
-      const R hh = odd ? tp.lo(2 * j + 1) : tp.lo(2 * j);
-      const R gg = odd ? tp.hi(2 * j + 1) : tp.hi(2 * j);
-      v2 += hh * cq[2 * cy][rk][kc - j] + gg * cq[2 * cy + 1][rk][kc - j];
+    for (int i = 0; i <= HK; ++i) {
+      q0[i] = cq[2 * cy][rk][kc + 1 - i];
+      q1[i] = cq[2 * cy + 1][rk][kc + 1 - i];
     }
-    tr[cy][rk][cl] = v2;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      R v2 = R(0);
+#pragma unroll
+      for (int j = 0; j < HK; ++j) {
+        const R hh = (u & 1) ? tp.lo(2 * j + 1) : tp.lo(2 * j);
+        const R gg = (u & 1) ? tp.hi(2 * j + 1) : tp.hi(2 * j);
+        v2 += hh * q0[j + 1 - (u >> 1)] + gg * q1[j + 1 - (u >> 1)];
+      }
+      tr[cy][rk][cl + u] = v2;
+    }
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < kTS * kTS; t += blockDim.x) {
-    const int ml = t / kTS, cl = t - ml * kTS;
-    const int m = m0 + ml, c = c0 + cl;
-    if (m >= n || c >= n) continue;
-    const bool odd = m & 1;
-    const int km = (m >> 1) - kb_m;
-    R v2 = R(0);
+  // columns: four adjacent output rows per thread likewise
+  static_assert(kTS * kTS == 4 * 256, "one group of four rows per thread");
+  {
+    const int cl = threadIdx.x % kTS, ml = (threadIdx.x / kTS) * 4;
+    const int c = c0 + cl;
+    const int km = (ml >> 1) + HK;
+    R q0[HK + 1], q1[HK + 1];
 #pragma unroll
-    for (int j = 0; j < K / 2; ++j) {
-      const R hh = odd ? tp.lo(2 * j + 1) : tp.lo(2 * j);
-      const R gg = odd ? tp.hi(2 * j + 1) : tp.hi(2 * j);
-      v2 += hh * tr[0][km - j][cl] + gg * tr[1][km - j][cl];
+    for (int i = 0; i <= HK; ++i) {
+      q0[i] = tr[0][km + 1 - i][cl];
+      q1[i] = tr[1][km + 1 - i][cl];
     }
-    out[(int64_t)m * ld + c] = v2;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int m = m0 + ml + u;
+      R v2 = R(0);
+#pragma unroll
+      for (int j = 0; j < HK; ++j) {
+        const R hh = (u & 1) ? tp.lo(2 * j + 1) : tp.lo(2 * j);
+        const R gg = (u & 1) ? tp.hi(2 * j + 1) : tp.hi(2 * j);
+        v2 += hh * q0[j + 1 - (u >> 1)] + gg * q1[j + 1 - (u >> 1)];
+      }
+      if (m < n && c < n) out[(int64_t)m * ld + c] = v2;
+    }
   }
   __syncthreads();
 }
