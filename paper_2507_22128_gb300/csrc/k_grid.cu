@@ -264,7 +264,25 @@ struct TileArgs {
   int64_t geom_off;
   int64_t ent_begin, ent_count;   // the partition's entries
   int* status;              // the job's status word (RIX_EINTERNAL on a failed check)
+  int slice, nsub;          // a work item is cut into nsub slices of `slice` entries (set_slices)
 };
+
+constexpr int kItemEntries = 2048;   // most entries of a work item (k_partition.cu)
+
+// How finely the work items are cut for `slots` resident CTAs.  A work item is
+// up to 2048 entries of one uv tile, so a small or centrally crowded
+// observation has a few long items and most SMs idle (19,841 samples at 128^2:
+// 207 us per gridding launch and 31 us per degridding, the time of one full
+// item; 17 and 5 us cut).  A slice is at most a quarter of a slot's share of
+// the entries, a power of two of at least 64: each slice stages and flushes
+// its tile, about the work of ten entries.
+void set_slices(TileArgs& a, int64_t slots) {
+  const int64_t share = a.ent_count / (4 * std::max<int64_t>(slots, 1));
+  int slice = 64;
+  while (slice < kItemEntries && slice < share) slice *= 2;
+  a.slice = slice;
+  a.nsub = kItemEntries / slice;
+}
 
 // On the PSF's 2N grid (x_psf = 2 x exactly), an image-grid tile of side T
 // at tx T maps to first taps in [2 tx T + 3, 2 tx T + 2 T + 2]: the staged
@@ -352,9 +370,13 @@ __global__ void __launch_bounds__(256) k_tiles(TileArgs a) {
   C* vout = static_cast<C*>(a.vis_out);
   const uint32_t tmask = (1u << a.bt) - 1u;
 
-  for (int64_t it = blockIdx.x; it < a.item_count; it += gridDim.x) {
-    const int64_t item = a.item_begin + it;
-    const uint32_t e0 = a.items[item], e1 = a.items[item + 1];
+  // entries a warp takes at a time: all eight warps share a short slice
+  const int wb = min(32, a.slice / nwarps);
+  for (int64_t it = blockIdx.x; it < a.item_count * a.nsub; it += gridDim.x) {
+    const int64_t item = a.item_begin + it / a.nsub;
+    const uint32_t e0 = a.items[item] + (uint32_t)((it % a.nsub) * a.slice);
+    const uint32_t e1 = min(a.items[item + 1], e0 + (uint32_t)a.slice);
+    if (e0 >= e1) continue;
     const uint32_t key = a.keys[e0];
     const int tx = (int)(key & tmask), ty = (int)((key >> a.bt) & tmask);
     const int p0 = (WW > 1) ? (int)((key >> (2 * a.bt)) & ((1u << a.bw) - 1u)) : 0;
@@ -375,8 +397,8 @@ __global__ void __launch_bounds__(256) k_tiles(TileArgs a) {
     }
     __syncthreads();
 
-    for (uint32_t base = e0 + warp * 32; base < e1; base += nwarps * 32) {
-      const int nvalid = (int)min(32u, e1 - base);
+    for (uint32_t base = e0 + warp * wb; base < e1; base += nwarps * wb) {
+      const int nvalid = (int)min((uint32_t)wb, e1 - base);
       const bool valid = lane < nvalid;
       // ---- per-lane sample geometry ----
       const uint32_t s = valid ? a.samples[base + lane] : 0u;
@@ -505,7 +527,7 @@ __global__ void __launch_bounds__(256) k_tiles(TileArgs a) {
 }
 
 template <typename R, int WW, int T, int MODE>
-int launch_tiles_impl(const Ctx* ctx, const TileArgs& a, cudaStream_t st) {
+int launch_tiles_impl(const Ctx* ctx, TileArgs a, cudaStream_t st) {
   using TG = TileGeom<T, MODE>;
   constexpr bool kUseModel = (MODE == kDegrid || MODE == kResid);
   constexpr bool kUseGrid = (MODE != kDegrid);
@@ -515,7 +537,9 @@ int launch_tiles_impl(const Ctx* ctx, const TileArgs& a, cudaStream_t st) {
   int per_sm = 0;
   RIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, sm));
   per_sm = std::max(per_sm, 1);
-  const int64_t blocks = std::min<int64_t>(a.item_count, (int64_t)ctx->num_sms * per_sm);
+  const int64_t slots = (int64_t)ctx->num_sms * per_sm;
+  set_slices(a, slots);
+  const int64_t blocks = std::min<int64_t>(a.item_count * a.nsub, slots);
   if (blocks <= 0) return RIX_OK;
   timing_mark(kTimeTiles, st, true);
   ::rix::note_launch(); kern<<<(unsigned)blocks, 256, sm, st>>>(a);
@@ -583,9 +607,11 @@ __global__ void __launch_bounds__(256) k_tiles_ws(TileArgs a) {
   const uint32_t tmask = (1u << a.bt) - 1u;
   const int per_warp = kWsBatch / nwarps;
 
-  for (int64_t it = blockIdx.x; it < a.item_count; it += gridDim.x) {
-    const int64_t item = a.item_begin + it;
-    const uint32_t e0 = a.items[item], e1 = a.items[item + 1];
+  for (int64_t it = blockIdx.x; it < a.item_count * a.nsub; it += gridDim.x) {
+    const int64_t item = a.item_begin + it / a.nsub;
+    const uint32_t e0 = a.items[item] + (uint32_t)((it % a.nsub) * a.slice);
+    const uint32_t e1 = min(a.items[item + 1], e0 + (uint32_t)a.slice);
+    if (e0 >= e1) continue;
     const uint32_t key = a.keys[e0];
     const int tx = (int)(key & tmask), ty = (int)((key >> a.bt) & tmask);
     const int p0 = (int)((key >> (2 * a.bt)) & ((1u << a.bw) - 1u));
@@ -723,7 +749,7 @@ __global__ void __launch_bounds__(256) k_tiles_ws(TileArgs a) {
 }
 
 template <typename R, int T, int MODE>
-int launch_tiles_ws(const Ctx* ctx, const TileArgs& a, cudaStream_t st) {
+int launch_tiles_ws(const Ctx* ctx, TileArgs a, cudaStream_t st) {
   using TG = WsGeom<T, MODE>;
   constexpr bool kUseModel = (MODE == kResid);
   const size_t sm = (size_t)(int(kUseModel) + 1) * kW * TG::PL * sizeof(cplx<R>) + kWsBatch * sizeof(WsRecord<R>);
@@ -732,7 +758,9 @@ int launch_tiles_ws(const Ctx* ctx, const TileArgs& a, cudaStream_t st) {
   int per_sm = 0;
   RIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, sm));
   per_sm = std::max(per_sm, 1);
-  const int64_t blocks = std::min<int64_t>(a.item_count, (int64_t)ctx->num_sms * per_sm);
+  const int64_t slots = (int64_t)ctx->num_sms * per_sm;
+  set_slices(a, slots);
+  const int64_t blocks = std::min<int64_t>(a.item_count * a.nsub, slots);
   if (blocks <= 0) return RIX_OK;
   timing_mark(kTimeTiles, st, true);
   ::rix::note_launch(); kern<<<(unsigned)blocks, 256, sm, st>>>(a);
