@@ -574,13 +574,8 @@ struct alignas(4 * sizeof(R)) WsRecord {
 };
 
 // header of a record as loaded by phase B
-static_assert(offsetof(WsRecord<float>, w) == 16 && sizeof(WsRecord<float>) % 16 == 0, "record layout");
 static_assert(offsetof(WsRecord<double>, w) == 32 && sizeof(WsRecord<double>) % 32 == 0, "record layout");
 template <typename R> struct WsHead { R yr, yi; uint32_t ouv; };
-__device__ __forceinline__ WsHead<float> ws_head(const WsRecord<float>& r) {
-  const float4 h = *reinterpret_cast<const float4*>(&r);
-  return {h.x, h.y, __float_as_uint(h.z)};
-}
 __device__ __forceinline__ WsHead<double> ws_head(const WsRecord<double>& r) {
   const double2 h = *reinterpret_cast<const double2*>(&r);
   return {h.x, h.y, r.ouv};
@@ -769,24 +764,23 @@ int launch_tiles_ws(const Ctx* ctx, TileArgs a, cudaStream_t st) {
   return RIX_OK;
 }
 
+// w-stacked jobs (tile 16): FP32 by register-resident footprints
+// (k_tiles_fp.cu; its PSF goes through launch_psf_fp), FP64 by the
+// plane-owned shared-memory sub-grid or, degridding, a warp per sample
 template <typename R, int MODE>
 int launch_tiles(const Job* job, const TileArgs& a, cudaStream_t st) {
-  const bool ws = job->nw > 0;
-  if constexpr (std::is_same<R, float>::value && (MODE == kGrid || MODE == kResid)) {
-    // FP32 w-stacked gridding on the image grid: register-resident
-    // footprints (k_tiles_fp.cu)
-    if (ws && job->tile == 16)
+  if (job->nw > 0) {
+    if constexpr (std::is_same<R, float>::value) {
       return launch_tiles_fp(job, MODE, a.item_begin, a.item_count, a.ent_begin, a.ent_count, a.win_lo, a.S, a.model,
-                             a.out, a.vis_in, st);
+                             a.out, a.vis_in, a.vis_out, st);
+    } else if constexpr (MODE == kDegrid) {
+      return launch_tiles_impl<R, kW, 16, MODE>(job->ctx, a, st);
+    } else {
+      return launch_tiles_ws<R, 16, MODE>(job->ctx, a, st);
+    }
   }
-  if constexpr (MODE != kDegrid) {
-    // w-stacked gridding: plane-owned shared-memory sub-grid (tile 16 only)
-    if (ws) return launch_tiles_ws<R, 16, MODE>(job->ctx, a, st);
-  }
-  if (job->tile == 16) {
-    return ws ? launch_tiles_impl<R, kW, 16, MODE>(job->ctx, a, st) : launch_tiles_impl<R, 1, 16, MODE>(job->ctx, a, st);
-  }
-  return ws ? launch_tiles_impl<R, kW, 32, MODE>(job->ctx, a, st) : launch_tiles_impl<R, 1, 32, MODE>(job->ctx, a, st);
+  if (job->tile == 16) return launch_tiles_impl<R, 1, 16, MODE>(job->ctx, a, st);
+  return launch_tiles_impl<R, 1, 32, MODE>(job->ctx, a, st);
 }
 
 TileArgs base_args(const Job* job, const Part& pt) {

@@ -17,9 +17,9 @@
 //     chunk into registers (lane: v row = lane & 7, planes lane >> 3 and that
 //     + 4, all 8 u taps: 16 complex cells, held as FP32 pairs of adjacent u
 //     taps),
-//   * per pair of samples forms the 2 x 24 kernel weights (one
-//     exponential-of-semicircle evaluation per weight, spread over the
-//     lanes), degrids both with packed FP32x2 FMAs, reduces them with a
+//   * forms the batch's kernel weights (24 exponential-of-semicircle
+//     evaluations per entry, spread over the lanes) and, per pair of samples,
+//     degrids both with packed FP32x2 FMAs, reduces them with a
 //     transposed butterfly (10 shuffles for the pair), forms the weighted
 //     residuals and spreads them into 16 complex accumulators per lane,
 //   * adds its accumulators into the shared-memory grid tile once per chunk,
@@ -30,6 +30,11 @@
 // mbarrier; the item's grid tile leaves by one TMA bulk reduce-add into the
 // partition's residual planes (element-wise atomic in L2), replacing
 // per-cell global atomics.  Tensor maps cover this GPU's own memory.
+//
+// kDegrid (rix_degrid) stops after the reduction and writes each sample's
+// model visibility; with no accumulators it takes four samples at a time.
+// The warp-per-sample k_tiles it replaced read every tap of every sample from
+// shared memory: 2.10 -> 1.27 ms for the 8.2 M entries of the 1024^2 job.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
@@ -371,22 +376,40 @@ struct FpArgs {
   const uint32_t* dev_items;   // grid mode: null, or the number of work items in device memory (item_count bounds it)
   int bt, bw, win_lo;
   int* status;                 // the job's status word
+  const uint32_t* samples;     // degrid: sample index per entry, gridder order
+  float2* vis_out;             // degrid: model visibility per sample
 };
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kGroup = 2;                     // samples degridded, reduced and gridded together
 constexpr int kCbMax = 1024;                  // chunk bounds of an item staged in shared memory
 
 // Exponential-of-semicircle weight of tap i (see es_weight) from the
 // hardware approximations: sqrt.approx and exp(x) = 2^(x log2 e) by
 // ex2.approx (relative errors near 2^-22, far below the FP32 operator's
 // 1e-5 bound).
-__device__ __forceinline__ float es_weight_fast(float d, int i) {
-  const float z = fmaf(d + (float)i, 2.0f / kW, -1.0f);
+__device__ __forceinline__ float es_weight_fast(float d, float i) {
+  const float z = fmaf(d + i, 2.0f / kW, -1.0f);
   const float t = fmaxf(fmaf(-z, z, 1.0f), 0.0f);
   float r, e;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(t));
   const float x = (float)(kBeta * 1.4426950408889634) * (r - 1.0f);
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x));
+  return e;
+}
+
+// The same with sqrt(1 - z^2) - 1 as -z^2 / (1 + sqrt(1 - z^2)): the root's
+// error no longer reaches the central taps' exponents undiminished (degridding
+// against the direct DFT 4e-7 instead of 8e-7 relative; 5e-7 with the IEEE root
+// and expf).  The other modes keep es_weight_fast: a major cycle's residual,
+// the difference of nearly equal terms, stays what it was.
+__device__ __forceinline__ float es_weight_acc(float d, float i) {
+  const float z = fmaf(d + i, 2.0f / kW, -1.0f);
+  const float zz = z * z;
+  const float t = fmaxf(fmaf(-z, z, 1.0f), 0.0f);
+  float r, q, e;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(t));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(1.0f + r));
+  const float x = ((float)(-kBeta * 1.4426950408889634) * zz) * q;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x));
   return e;
 }
@@ -427,12 +450,15 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 
-// per warp: two chunk slots ({du, dv, dw, tap} and {w re v, w im v, w, 0} of
-// up to 32 entries) and the weights of one group of samples
+// per warp: a batch's records ({du, dv, dw, tap}; {w re v, w im v, w, 0}, the
+// next batch's beside it) and its kernel weights, 24 per entry (8 u, 8 v, 8 w).
+// The weights are formed once per batch: formed per pair of entries instead
+// (48 over 64 lane slots) they cost 10 instructions per entry rather than 6-7
+// and put a square root and an exponential at the head of every pair's chain.
 struct WarpScratch {
-  float4 g[2][kChunkMax];
+  float4 g[kChunkMax];
   float4 y[2][kChunkMax];
-  float w[kGroup * 24];
+  float w[kChunkMax * 24];
 };
 
 // Several partitions (of one or more jobs) in one launch: per pair its
@@ -450,7 +476,12 @@ template <int MODE, bool BATCH>
 __global__ void __launch_bounds__(kFpThreads, 2)
     k_tiles_fp(FpArgs a0, const __grid_constant__ CUtensorMap tm_model0, const __grid_constant__ CUtensorMap tm_out0,
                FpBatch bt) {
-  constexpr bool kModel = (MODE == kResid);
+  constexpr bool kModel = (MODE != kGrid);
+  constexpr bool kSpread = (MODE != kDegrid);
+  // samples degridded, reduced and gridded together: four only where the
+  // registers of one CTA pair per SM allow it (degridding 1.38 -> 1.27 ms for
+  // 8.2 M entries; with the accumulators beside the model it spills)
+  constexpr int kGroup = MODE == kDegrid ? 4 : 2;
   __shared__ FpArgs sa;   // the arguments of the pair the CTA works on
   if (!BATCH && threadIdx.x == 0) sa = a0;
   const FpArgs& a = sa;
@@ -458,8 +489,8 @@ __global__ void __launch_bounds__(kFpThreads, 2)
   unsigned char* base =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
   float* grid = reinterpret_cast<float*>(base);
-  const float2* model = reinterpret_cast<const float2*>(base + kTileBytes);
-  unsigned char* tail = base + (kModel ? 2 : 1) * kTileBytes;
+  const float2* model = reinterpret_cast<const float2*>(base + (kSpread ? kTileBytes : 0));
+  unsigned char* tail = base + (int(kModel) + int(kSpread)) * kTileBytes;
   WarpScratch* scratch = reinterpret_cast<WarpScratch*>(tail);
   uint32_t* cb = reinterpret_cast<uint32_t*>(scratch + kFpWarps);   // chunk bounds of the item
   uint32_t* queue = cb + kCbMax;                                     // next chunk to claim
@@ -468,8 +499,8 @@ __global__ void __launch_bounds__(kFpThreads, 2)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int vrow = lane & 7, pa = lane >> 3;         // this lane's v row and planes pa, pa + 4
-  const int mine = (lane >> 4) & 1;                  // the group sample whose degrid sum this lane ends with
-  const bool b4 = (lane >> 4) & 1;
+  const bool b4 = (lane >> 4) & 1, b3 = (lane >> 3) & 1;
+  const int mine = kGroup == 4 ? 2 * int(b3) + int(b4) : int(b4);   // the group sample whose degrid sum this lane ends with
   const uint32_t bar_a = smem_u32(bar);
   if (threadIdx.x == 0) *lock = 0u;
   if (kModel && threadIdx.x == 0) {
@@ -480,7 +511,6 @@ __global__ void __launch_bounds__(kFpThreads, 2)
   __syncthreads();
   uint32_t phase = 0;
   WarpScratch& ws = scratch[warp];
-  float* wg = ws.w;
 
   int64_t total = BATCH ? bt.item_start[bt.n] : a0.item_count;
   if constexpr (MODE == kGrid && !BATCH) {
@@ -526,7 +556,8 @@ __global__ void __launch_bounds__(kFpThreads, 2)
     const uint32_t c0 = a.item_chunk[item];
     const int nch = (int)(a.item_chunk[item + 1] - c0);
     float4* g4 = reinterpret_cast<float4*>(grid);
-    for (int i = threadIdx.x; i < kTileFloats / 4; i += kFpThreads) g4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if constexpr (kSpread)
+      for (int i = threadIdx.x; i < kTileFloats / 4; i += kFpThreads) g4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int i = threadIdx.x; i <= nch && i < kCbMax; i += kFpThreads) cb[i] = a.chunks[c0 + i];
     if (threadIdx.x == 0) *queue = 0u;
     if (kModel) {
@@ -560,15 +591,16 @@ __global__ void __launch_bounds__(kFpThreads, 2)
       if (lane == 0) k = (int)atomicAdd(queue, 1u);
       return __shfl_sync(kFull, k, 0);
     };
-    // start the copies of the nb (<= 32) entries from eb into slot `sl`;
-    // slot entries past nb are zero (zero weight and data)
+    // start the copies of the nb (<= 32) entries from eb: the geometry into
+    // the one slot (its last batch's weights are formed), the visibilities
+    // into slot `sl`; entries past nb are zero (zero weight and data)
     auto fetch = [&](uint32_t eb, int nb, int sl) {
       if (lane < nb) {
-        cp_async16(&ws.g[sl][lane], a.geom + eb + lane);
-        cp_async16(&ws.y[sl][lane], a.ysamp + eb + lane);
+        cp_async16(&ws.g[lane], a.geom + eb + lane);
+        if constexpr (kSpread) cp_async16(&ws.y[sl][lane], a.ysamp + eb + lane);
       } else {
-        ws.g[sl][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-        ws.y[sl][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+        ws.g[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if constexpr (kSpread) ws.y[sl][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -597,6 +629,48 @@ __global__ void __launch_bounds__(kFpThreads, 2)
       bool first = true, more = true;
       while (more) {
         const int nb = (int)min(end - pos, 32u);
+        // this batch's records have landed: its kernel weights
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncwarp();
+        const uint32_t ouv = __float_as_uint(ws.g[0].w);
+        {
+          if constexpr (MODE == kResid) {
+            // an entry per lane (fewer registers live in the residual mode:
+            // 11.14 against 11.45 ms for ten launches of the 1024^2 job, where
+            // the gridding mode takes 1.97 against 1.86 ms)
+            const float4 g = ws.g[lane];
+            const float d[3] = {g.x, g.y, g.z};
+            float4* wl = reinterpret_cast<float4*>(ws.w + lane * 24);
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+              const float t0 = (float)(4 * (q & 1));
+              wl[q] = make_float4(es_weight_fast(d[q >> 1], t0), es_weight_fast(d[q >> 1], t0 + 1.f),
+                                  es_weight_fast(d[q >> 1], t0 + 2.f), es_weight_fast(d[q >> 1], t0 + 3.f));
+            }
+          } else {
+            // four entries at a time: lane = (entry, tap), the three axes in turn
+            const int nb4 = (nb + 3) & ~3;
+            const float fi = (float)(lane & 7);
+#pragma unroll 2
+            for (int r = lane >> 3; r < nb4; r += 4) {
+              const float4 g = ws.g[r];
+              float* wr = ws.w + r * 24 + (lane & 7);
+              if constexpr (MODE == kDegrid) {
+                wr[0] = es_weight_acc(g.x, fi);
+                wr[8] = es_weight_acc(g.y, fi);
+                wr[16] = es_weight_acc(g.z, fi);
+              } else {
+                wr[0] = es_weight_fast(g.x, fi);
+                wr[8] = es_weight_fast(g.y, fi);
+                wr[16] = es_weight_fast(g.z, fi);
+              }
+            }
+          }
+        }
+        uint32_t smp = 0;   // degrid: the lane's entry's sample
+        if constexpr (!kSpread)
+          if (lane < nb) smp = a.samples[pos + lane];
+        __syncwarp();
         // the next batch: the rest of this chunk, else the next chunk's first
         npos = pos + (uint32_t)nb;
         more = npos < end;
@@ -609,18 +683,10 @@ __global__ void __launch_bounds__(kFpThreads, 2)
             next = true;
           }
         }
-        if (next) {
-          fetch(npos, (int)min(nend - npos, 32u), sl ^ 1);
-          asm volatile("cp.async.wait_group 1;" ::: "memory");
-        } else {
-          asm volatile("cp.async.wait_group 0;" ::: "memory");
-        }
-        __syncwarp();
-        const float4* sd = ws.g[sl];
+        if (next) fetch(npos, (int)min(nend - npos, 32u), sl ^ 1);
         const float4* sy = ws.y[sl];
         if (first) {
           first = false;
-          const uint32_t ouv = __float_as_uint(sd[0].w);
           cell = (int)(ouv & 0xffu) * kRow + (int)(ouv >> 8) + vrow;   // complex cell in a plane
           if (kModel) {
 #pragma unroll
@@ -637,17 +703,7 @@ __global__ void __launch_bounds__(kFpThreads, 2)
           }
         }
         for (int j0 = 0; j0 < nb; j0 += kGroup) {
-          // ---- the group's kGroup x 24 kernel weights over the warp's lanes:
-          // entry e of sample e / 24, tap e % 24 (0-7 u, 8-15 v, 16-23 w)
-#pragma unroll
-          for (int r = 0; r < (kGroup * 24 + 31) / 32; ++r) {
-            const int e = lane + 32 * r;
-            if (e >= kGroup * 24) break;
-            const int kk = e / 24, tap = e - 24 * (e / 24);
-            const float* dk = reinterpret_cast<const float*>(&sd[j0 + kk]);
-            wg[e] = es_weight_fast(dk[tap >> 3], tap & 7);
-          }
-          __syncwarp();
+          const float* wg = ws.w + j0 * 24;
           // per sample: the lane's v-row times w-plane weights (fa: plane pa,
           // fb: plane pa + 4)
           float fa[kGroup], fb[kGroup];
@@ -681,26 +737,36 @@ __global__ void __launch_bounds__(kFpThreads, 2)
             // pair, so the lane ends with the sum over all 32 lanes of sample
             // `mine` after 10 shuffles for the 2 samples
             float2 tot = bfly(b4, part[0], part[1], 16);
-            tot.x += __shfl_xor_sync(kFull, tot.x, 8);
-            tot.y += __shfl_xor_sync(kFull, tot.y, 8);
+            if constexpr (kGroup == 4) {
+              tot = bfly(b3, tot, bfly(b4, part[2], part[3], 16), 8);
+            } else {
+              tot.x += __shfl_xor_sync(kFull, tot.x, 8);
+              tot.y += __shfl_xor_sync(kFull, tot.y, 8);
+            }
             tot.x += __shfl_xor_sync(kFull, tot.x, 4);
             tot.y += __shfl_xor_sync(kFull, tot.y, 4);
             tot.x += __shfl_xor_sync(kFull, tot.x, 2);
             tot.y += __shfl_xor_sync(kFull, tot.y, 2);
             tot.x += __shfl_xor_sync(kFull, tot.x, 1);
             tot.y += __shfl_xor_sync(kFull, tot.y, 1);
-            const float4 ym = sy[j0 + mine];
-            y0 = fmaf(-ym.z, tot.x, ym.x);
-            y1 = fmaf(-ym.z, tot.y, ym.y);
+            if constexpr (kSpread) {
+              const float4 ym = sy[j0 + mine];
+              y0 = fmaf(-ym.z, tot.x, ym.x);
+              y1 = fmaf(-ym.z, tot.y, ym.y);
+            } else {
+              const uint32_t s0 = __shfl_sync(kFull, smp, j0 + mine);
+              if ((lane & (kGroup == 4 ? 7 : 15)) == 0 && j0 + mine < nb) a.vis_out[s0] = tot;
+            }
           }
+          if constexpr (!kSpread) continue;
           // ---- grid the group's samples into the accumulators
 #pragma unroll
           for (int kk = 0; kk < kGroup; ++kk) {
             const float fak = fa[kk], fbk = fb[kk];
             float yrk, yik;
             if (kModel) {
-              yrk = __shfl_sync(kFull, y0, 16 * kk);
-              yik = __shfl_sync(kFull, y1, 16 * kk);
+              yrk = __shfl_sync(kFull, y0, 16 * (kk & 1) + 8 * (kk >> 1));
+              yik = __shfl_sync(kFull, y1, 16 * (kk & 1) + 8 * (kk >> 1));
             } else {
               const float4 yk = sy[j0 + kk];
               yrk = yk.x;
@@ -719,12 +785,12 @@ __global__ void __launch_bounds__(kFpThreads, 2)
               abi[t] = ffma2(cbi, wu[t], abi[t]);
             }
           }
-          __syncwarp();   // the group's weights are read before the next group overwrites them
         }
-        __syncwarp();   // the slot is read before its next fetch
+        __syncwarp();   // the weights and the slot are read before they are overwritten
         sl ^= 1;
         if (more) pos = npos;
       }
+      if constexpr (kSpread) {
       // add the chunk's accumulators into the item's grid tile: plain
       // read-modify-writes under the CTA's flush lock (the chunks of one
       // item overlap; with shared-memory float atomics instead, a launch of
@@ -765,17 +831,20 @@ __global__ void __launch_bounds__(kFpThreads, 2)
         __threadfence_block();
         if (held) atomicExch(lock, 0u);
       }
+      }
       k = k2;
       pos = npos;
       end = nend;
     }
     // the grid tile's shared-memory writes become visible to the TMA unit,
     // then one thread adds the tile into the residual planes
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      tma_reduce_add_3d(tm_out, 2 * v0, u0, p0, smem_u32(grid));
-      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    if constexpr (kSpread) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        tma_reduce_add_3d(tm_out, 2 * v0, u0, p0, smem_u32(grid));
+        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+      }
     }
     __syncthreads();
   }
@@ -892,12 +961,18 @@ int gather_y(const Job* job, int64_t ent_begin, int64_t ent_count, const void* v
 
 int launch_tiles_fp(const Job* job, int mode, int64_t item_begin, int64_t item_count, int64_t ent_begin,
                     int64_t ent_count, int win_lo, int S, const void* model_planes, void* out_planes, const void* vis,
-                    cudaStream_t st) {
+                    void* vis_out, cudaStream_t st) {
   if (item_count <= 0 || ent_count <= 0) return RIX_OK;
-  if (job->tile != kT || job->nw < kW || job->fp64 || (mode != kGrid && mode != kResid) || (S & 1))
+  if (job->tile != kT || job->nw < kW || job->fp64 || (mode != kGrid && mode != kResid && mode != kDegrid) || (S & 1))
     return set_error(RIX_EINVAL, "k_tiles_fp: unsupported job (tile %d, planes %d)", job->tile, job->nw);
-  const FpArgs a = fp_args(job, item_begin, item_count, win_lo);
+  FpArgs a = fp_args(job, item_begin, item_count, win_lo);
   CUtensorMap tm_out, tm_model;
+  if (mode == kDegrid) {
+    a.samples = job->gsamples.as<uint32_t>();
+    a.vis_out = static_cast<float2*>(vis_out);
+    RIX_TRY(plane_map(&tm_model, model_planes, S, job->nw));
+    return launch_fp<kDegrid>(job, a, tm_model, tm_model, st);
+  }
   RIX_TRY(plane_map(&tm_out, out_planes, S, job->nw));
   // the weighted visibilities of the partition's entries in gridder order
   RIX_TRY(gather_y(job, ent_begin, ent_count, vis, st));

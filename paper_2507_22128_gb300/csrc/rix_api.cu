@@ -864,7 +864,7 @@ int rix_gridder_probe(rix_job_t job, int part, const void* vis_obs, int32_t reps
   if (rc == RIX_OK && cudaEventRecord(e0, st) != cudaSuccess) rc = set_error(RIX_ECUDA, "event");
   for (int r = 0; r < reps && rc == RIX_OK; ++r)
     rc = launch_tiles_fp(&J, kResid, pt.item_begin, pt.item_count, pt.ent_begin, pt.ent_count, pt.win_lo, pt.win_n,
-                         pt.model_planes.p, pt.resid_planes.p, vis_obs, st);
+                         pt.model_planes.p, pt.resid_planes.p, vis_obs, nullptr, st);
   float ms = 0.f;
   if (rc == RIX_OK && (cudaEventRecord(e1, st) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
                        cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))

@@ -403,12 +403,13 @@ template <typename R>
 int grid_work_order(Job* job, cudaStream_t st);
 // The FP32 w-stacked gridder with register-resident kernel footprints
 // (k_tiles_fp.cu): mode kGrid spreads w * vis into out_planes, kResid
-// degrids model_planes and spreads w * (vis - model visibility); planes
+// degrids model_planes and spreads w * (vis - model visibility), kDegrid
+// writes the model visibilities to vis_out; planes
 // [n_wplanes][S][S] complex on the partition's uv window [win_lo, win_lo + S)
 // (out_planes zeroed by the caller).  Tile side 16.
 int launch_tiles_fp(const Job* job, int mode, int64_t item_begin, int64_t item_count, int64_t ent_begin,
                     int64_t ent_count, int win_lo, int S, const void* model_planes, void* out_planes, const void* vis,
-                    cudaStream_t st);
+                    void* vis_out, cudaStream_t st);
 // The PSF gridding of partition p on the same gridder (FP32 w-stacked jobs
 // with tile 16): unit visibilities times the weights spread on the PSF grid
 // (coordinate x = u_lambda * scale + half) into planes [n_wplanes][S][S]
