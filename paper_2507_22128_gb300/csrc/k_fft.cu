@@ -24,17 +24,29 @@ namespace rix {
 namespace {
 
 // screen[p][pix] = corr[pix] * exp(-2 pi i (w0 + p dw) nm1[pix]), formed as
-// the row passes form it (wscreen)
+// the row passes form it (wscreen).  n - 1 and corr are even in both
+// coordinates: one thread per quadrant pixel of a plane forms the phase (FP64)
+// once for the up to four pixels that share it.
 template <typename R>
-__global__ void k_screen_table(int64_t npix, int nplanes, double w0, double dw, const R* __restrict__ corr,
+__global__ void k_screen_table(int M, int nplanes, double w0, double dw, const R* __restrict__ corr,
                                const double* __restrict__ nm1, cplx<R>* __restrict__ screen) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < npix * nplanes;
+  const int h = M / 2;
+  const int64_t q = (int64_t)(h + 1) * (h + 1), npix = (int64_t)M * M;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < q * nplanes;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const int p = (int)(i / npix);
-    const int64_t pix = i - (int64_t)p * npix;
+    const int p = (int)(i / q);
+    const int r = (int)(i - p * q), b = r / (h + 1), c = r - b * (h + 1);
+    const int64_t pix = (int64_t)b * M + c;
     const cplx<R> e = wscreen<R, -1>(w0 + p * dw, nm1[pix]);
-    const R c = corr[pix];
-    screen[i] = cmake<cplx<R>>(e.x * c, e.y * c);
+    const R f = corr[pix];
+    const cplx<R> z = cmake<cplx<R>>(e.x * f, e.y * f);
+    cplx<R>* s = screen + p * npix;
+    const int bm = M - b, cm = M - c;     // the mirrors of h - b and h - c
+    const bool mb = b > 0 && b < h, mc = c > 0 && c < h;
+    s[pix] = z;
+    if (mc) s[(int64_t)b * M + cm] = z;
+    if (mb) s[(int64_t)bm * M + c] = z;
+    if (mb && mc) s[(int64_t)bm * M + cm] = z;
   }
 }
 
@@ -79,9 +91,9 @@ int build_screen_table(const Ctx* ctx, const XformGeom& g, cplx<R>* screen, cuda
   if (g.mode != kFacPhase || !g.corr || !g.nm1 || g.M <= 0 || g.nplanes <= 0)
     return set_error(RIX_EINVAL, "screen table needs a w-stacked geometry");
   const int64_t npix = (int64_t)g.M * g.M;
-  const int blocks = (int)std::min<int64_t>(ceil_div(npix * g.nplanes, 256), (int64_t)ctx->num_sms * 16);
+  const int blocks = (int)std::min<int64_t>(ceil_div(npix * g.nplanes, 4 * 256), (int64_t)ctx->num_sms * 16);
   ::rix::note_launch();
-  k_screen_table<R><<<blocks, 256, 0, st>>>(npix, g.nplanes, g.w0, g.dw, static_cast<const R*>(g.corr), g.nm1,
+  k_screen_table<R><<<blocks, 256, 0, st>>>(g.M, g.nplanes, g.w0, g.dw, static_cast<const R*>(g.corr), g.nm1,
                                             screen);
   RIX_LAUNCH_CHECK();
   return RIX_OK;

@@ -55,11 +55,12 @@ void gauss_legendre(int n, std::vector<double>& x, std::vector<double>& w) {
 // Fourier transform of the ES kernel over cell units,
 //   Phi(f) = (W/2) int_{-1}^{1} phi(z) cos(pi W z f) dz,
 // with z = sin(t) (analytic integrand), by Gauss-Legendre quadrature in t.
+constexpr int kEsNodes = 96;
 struct EsFourier {
   std::vector<double> st, wt;
   EsFourier() {
     std::vector<double> x, w;
-    gauss_legendre(96, x, w);
+    gauss_legendre(kEsNodes, x, w);
     st.resize(x.size());
     wt.resize(x.size());
     for (size_t k = 0; k < x.size(); ++k) {
@@ -74,6 +75,28 @@ struct EsFourier {
     return 0.5 * kW * acc;
   }
 };
+
+// the same quadrature for the M pixels of a table, a warp per value: 1 / Phi(
+// (a - M/2) / ng).  On the host the two tables of a 1024^2 job took 295,000
+// cosines, 2.4 ms of a 12.7 ms set-up during which the GPU idled.
+struct EsNodes {
+  double st[kEsNodes], wt[kEsNodes];
+};
+__global__ void k_es_fourier(const __grid_constant__ EsNodes nodes, int M, int ng, double* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const int warps = (gridDim.x * blockDim.x) >> 5;
+  for (int a = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; a <= M / 2; a += warps) {
+    const double f = (double)(a - M / 2) / ng;
+    double acc = 0.0;
+    for (int k = lane; k < kEsNodes; k += 32) acc += nodes.wt[k] * cospi((double)kW * f * nodes.st[k]);
+    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) {
+      const double v = 1.0 / (0.5 * kW * acc);
+      out[a] = v;
+      if (a > 0 && M - a < M) out[M - a] = v;   // Phi is even
+    }
+  }
+}
 
 // Chebyshev coefficients of Phi on [lo, hi] (degree kCheb - 1): Phi is entire
 // and |pi W f| <= 2 pi over the w-correction's range, so 40 terms reach
@@ -95,47 +118,12 @@ struct CorrArgs {
   int M;
   int ox, oy;           // pixel offset of the table's centre from the phase centre
   double cell;
-  const double* p1;     // Phi((a - M/2) / Ng), [M]
+  const double* ip1;    // 1 / Phi((a - M/2) / Ng), [M]
   int wstack;
   double dw, lo, hi;    // Chebyshev interval of dw (n - 1)
+  int ncheb;            // leading coefficients that count
   double cheb[kCheb];
 };
-
-// corr[b][a] = 1 / (Phi(a'/Ng) Phi(b'/Ng) [n Phi(dw (n-1))]),  nm1[b][a] = n - 1,
-// with a' = a - M/2, b' = b - M/2 the offsets from the table's centre and n at
-// the sky position (a' + ox, b' + oy) cells from the phase centre
-template <typename R>
-__global__ void k_corrections(CorrArgs a, R* __restrict__ corr, double* __restrict__ nm1) {
-  const int64_t tot = (int64_t)a.M * a.M;
-  const int h = a.M / 2;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(i / a.M), c = (int)(i - (int64_t)b * a.M);
-    double v = 1.0 / (a.p1[c] * a.p1[b]);
-    if (a.wstack) {
-      const double l = (double)(c - h + a.ox) * a.cell, m = (double)(b - h + a.oy) * a.cell;
-      const double r2 = __dadd_rn(__dmul_rn(l, l), __dmul_rn(m, m));
-      const double n = __dsqrt_rn(1.0 - r2);
-      const double d = -r2 / (1.0 + n);
-      double phw;
-      if (a.hi > a.lo) {
-        // Clenshaw recurrence for sum_j c_j T_j(x)
-        const double x = (2.0 * a.dw * d - (a.lo + a.hi)) / (a.hi - a.lo);
-        double b1 = 0.0, b2 = 0.0;
-        for (int j = kCheb - 1; j >= 1; --j) {
-          const double t = 2.0 * x * b1 - b2 + a.cheb[j];
-          b2 = b1;
-          b1 = t;
-        }
-        phw = x * b1 - b2 + a.cheb[0];
-      } else {
-        phw = a.cheb[0];
-      }
-      v /= n * phw;
-      nm1[i] = d;
-    }
-    corr[i] = (R)v;
-  }
-}
 
 // dw (n - 1) -> n Phi(dw (n - 1)) and n - 1 at squared radius r2 (a Clenshaw
 // sum of the Chebyshev fit of Phi)
@@ -146,7 +134,7 @@ __device__ __forceinline__ double wfactor(const CorrArgs& a, double r2, double* 
   if (a.hi > a.lo) {
     const double x = (2.0 * a.dw * d - (a.lo + a.hi)) / (a.hi - a.lo);
     double b1 = 0.0, b2 = 0.0;
-    for (int j = kCheb - 1; j >= 1; --j) {
+    for (int j = a.ncheb - 1; j >= 1; --j) {
       const double t = 2.0 * x * b1 - b2 + a.cheb[j];
       b2 = b1;
       b1 = t;
@@ -159,6 +147,26 @@ __device__ __forceinline__ double wfactor(const CorrArgs& a, double r2, double* 
   return n * phw;
 }
 
+// corr[b][a] = 1 / (Phi(a'/Ng) Phi(b'/Ng) [n Phi(dw (n-1))]),  nm1[b][a] = n - 1,
+// with a' = a - M/2, b' = b - M/2 the offsets from the table's centre and n at
+// the sky position (a' + ox, b' + oy) cells from the phase centre
+template <typename R>
+__global__ void k_corrections(CorrArgs a, R* __restrict__ corr, double* __restrict__ nm1) {
+  const int64_t tot = (int64_t)a.M * a.M;
+  const int h = a.M / 2;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (int64_t)gridDim.x * blockDim.x) {
+    const int b = (int)(i / a.M), c = (int)(i - (int64_t)b * a.M);
+    double v = a.ip1[c] * a.ip1[b];
+    if (a.wstack) {
+      const double l = (double)(c - h + a.ox) * a.cell, m = (double)(b - h + a.oy) * a.cell;
+      double d;
+      v /= wfactor(a, __dadd_rn(__dmul_rn(l, l), __dmul_rn(m, m)), &d);
+      nm1[i] = d;
+    }
+    corr[i] = (R)v;
+  }
+}
+
 // k_corrections for a table centred on the phase centre (ox = oy = 0): the
 // w-factor depends on l^2 + m^2 only, so one thread per pixel of the quadrant
 // [0, M/2]^2 evaluates it once and writes the up to four pixels (b, c),
@@ -169,10 +177,10 @@ __global__ void k_corrections_sym(CorrArgs a, R* __restrict__ corr, double* __re
   const int64_t q = (int64_t)(h + 1) * (h + 1);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < q; i += (int64_t)gridDim.x * blockDim.x) {
     const int b = (int)(i / (h + 1)), c = (int)(i - (int64_t)b * (h + 1));
-    double wf = 1.0, d = 0.0;
+    double d = 0.0, v = a.ip1[c] * a.ip1[b];   // even in b - h and c - h
     if (a.wstack) {
       const double l = (double)(c - h) * a.cell, m = (double)(b - h) * a.cell;
-      wf = wfactor(a, __dadd_rn(__dmul_rn(l, l), __dmul_rn(m, m)), &d);
+      v /= wfactor(a, __dadd_rn(__dmul_rn(l, l), __dmul_rn(m, m)), &d);
     }
     const int bs[2] = {b, 2 * h - b}, cs[2] = {c, 2 * h - c};
     for (int u = 0; u < 2; ++u) {
@@ -182,7 +190,7 @@ __global__ void k_corrections_sym(CorrArgs a, R* __restrict__ corr, double* __re
         const int cc = cs[w];
         if (cc >= a.M || (w == 1 && cc == c)) continue;
         const int64_t pix = (int64_t)bb * a.M + cc;
-        corr[pix] = (R)(1.0 / (a.p1[cc] * a.p1[bb] * wf));
+        corr[pix] = (R)v;
         if (a.wstack) nm1[pix] = d;
       }
     }
@@ -197,8 +205,6 @@ int fill_correction(Job* job, int M, int ng, int ox, int oy, int half_px, R* cor
   static const EsFourier phi;
   const bool ws = job->nw > 0;
   const double cell = job->desc.cell_rad, dw = job->stats.dw;
-  std::vector<double> p1(M);
-  for (int a = 0; a < M; ++a) p1[a] = phi((double)(a - M / 2) / ng);
   CorrArgs ca{};
   ca.M = M;
   ca.ox = ox;
@@ -216,20 +222,26 @@ int fill_correction(Job* job, int M, int ng, int ox, int oy, int half_px, R* cor
     ca.hi = 0.0;
     if (ca.hi > ca.lo) chebyshev_fit(phi, ca.lo, ca.hi, ca.cheb);
     else ca.cheb[0] = phi(0.0);
+    // the trailing coefficients below 1e-19 of the first do not reach a double's
+    // rounding (about a dozen of the 40 do at the usual plane spacings)
+    for (ca.ncheb = kCheb; ca.ncheb > 1 && std::fabs(ca.cheb[ca.ncheb - 1]) < 1e-19 * std::fabs(ca.cheb[0]);) --ca.ncheb;
     job->stats.max_dw_nm1 = std::max(job->stats.max_dw_nm1, std::fabs(dmin));
   }
-  double* p1d = nullptr;
-  RIX_CUDA(::rix::malloc_async((void**)&p1d, M * sizeof(double), st));
-  RIX_CUDA(cudaMemcpyAsync(p1d, p1.data(), M * sizeof(double), cudaMemcpyHostToDevice, st));
-  ca.p1 = p1d;
+  double* ip1 = nullptr;
+  RIX_CUDA(::rix::malloc_async((void**)&ip1, M * sizeof(double), st));
+  EsNodes nodes;
+  std::copy(phi.st.begin(), phi.st.end(), nodes.st);
+  std::copy(phi.wt.begin(), phi.wt.end(), nodes.wt);
+  ::rix::note_launch();
+  k_es_fourier<<<(unsigned)ceil_div(M / 2 + 1, 8), 256, 0, st>>>(nodes, M, ng, ip1);
+  ca.ip1 = ip1;
   const int64_t tot = (int64_t)M * M;
   const int blocks = (int)std::min<int64_t>(ceil_div(tot, 256), (int64_t)job->ctx->num_sms * 16);
   ::rix::note_launch();
   if (ox == 0 && oy == 0) k_corrections_sym<R><<<blocks, 256, 0, st>>>(ca, corr, ws ? nm1 : nullptr);
   else k_corrections<R><<<blocks, 256, 0, st>>>(ca, corr, ws ? nm1 : nullptr);
-  cudaFreeAsync(p1d, st);
+  cudaFreeAsync(ip1, st);
   RIX_LAUNCH_CHECK();
-  RIX_CUDA(cudaStreamSynchronize(st));   // p1 is a host temporary
   return RIX_OK;
 }
 
@@ -252,7 +264,7 @@ struct TileArgs {
   int nchan;
   double scale, half;       // grid coordinate x = u_l * scale + half
   int nw, ww;
-  double w_min, dw;
+  double w_min, dw, inv_dw;
   int bt, bw, logT;
   int win_lo, S;            // plane window [win_lo, win_lo + S)^2
   const void* model;        // cplx [planes][S][S], u-major
@@ -329,7 +341,7 @@ __global__ void k_entry_geom(TileArgs a, int64_t e_off, int64_t n, EntryGeom<R>*
     g.dw = R(0);
     if (a.nw > 0) {
       const double wl = __dmul_rn(a.uvw[row * 3 + 2], sc);
-      const double tw = __ddiv_rn(__dadd_rn(wl, -a.w_min), a.dw);
+      const double tw = div_by(__dadd_rn(wl, -a.w_min), a.dw, a.inv_dw);
       const double pc = fmin(fmax(ceil(tw), 0.0), (double)(a.nw - a.ww));
       g.dw = (R)__dadd_rn(pc, -tw);
     }
@@ -799,6 +811,7 @@ TileArgs base_args(const Job* job, const Part& pt) {
   a.ww = job->ww;
   a.w_min = job->stats.w_min;
   a.dw = job->stats.dw;
+  a.inv_dw = exact_reciprocal(job->stats.dw);
   a.bt = job->bt;
   a.bw = job->bw;
   a.logT = ilog2(job->tile);

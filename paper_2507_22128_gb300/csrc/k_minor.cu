@@ -78,19 +78,28 @@ __device__ __forceinline__ double ramp(double ell, double delta, double r) {
   return fmin(fmax((ell + delta - r) / (2.0 * delta), 0.0), 1.0);
 }
 
+// one thread per quadrant value (|k_u|, |k_v|) writes the up to four entries
+// that share its radius (FP64 root and quotients bound it)
 template <typename R>
 __global__ void k_gamma(GammaArgs a, R* __restrict__ gam) {
-  const int L = 2 * a.n;
-  const int64_t tot = (int64_t)L * L;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (int64_t)gridDim.x * blockDim.x) {
-    const int ju = (int)(i / L), jv = (int)(i - (int64_t)ju * L);
-    const double ku = ju - a.n, kv = jv - a.n;
-    const double r = sqrt(ku * ku + kv * kv) / 2.0;
+  const int n = a.n, L = 2 * a.n;
+  const int64_t tot = (int64_t)L * L, q = (int64_t)(n + 1) * (n + 1);
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < q; i += (int64_t)gridDim.x * blockDim.x) {
+    const int ku = (int)(i / (n + 1)), kv = (int)(i - (int64_t)ku * (n + 1));
+    const double du = ku, dv = kv;
+    const double r = sqrt(du * du + dv * dv) / 2.0;
     double lam_lo = 0.0;
     for (int p = 0; p < a.nparts; ++p) {
       const double lam_hi = (p == a.nparts - 1) ? 1.0 : ramp(a.ells[p], a.delta, r);
-      gam[(int64_t)p * tot + i] = (R)(lam_hi - lam_lo);
+      const R v = (R)(lam_hi - lam_lo);
       lam_lo = lam_hi;
+      R* g = gam + (int64_t)p * tot;
+      // indices n - k and n + k (k = n has no positive index)
+      const bool pu = ku > 0 && ku < n, pv = kv > 0 && kv < n;
+      g[(int64_t)(n - ku) * L + n - kv] = v;
+      if (pv) g[(int64_t)(n - ku) * L + n + kv] = v;
+      if (pu) g[(int64_t)(n + ku) * L + n - kv] = v;
+      if (pu && pv) g[(int64_t)(n + ku) * L + n + kv] = v;
     }
   }
 }
@@ -632,7 +641,7 @@ int fill_init(Job* job, cudaStream_t st) {
   ga.nparts = P;
   for (int i = 0; i < P - 1; ++i) ga.ells[i] = job->ells[i];
   ga.delta = job->stats.delta_px;
-  ::rix::note_launch(); k_gamma<R><<<blocks_for(job->ctx, tot), 256, 0, st>>>(ga, job->gam.as<R>());
+  ::rix::note_launch(); k_gamma<R><<<blocks_for(job->ctx, (int64_t)(n + 1) * (n + 1)), 256, 0, st>>>(ga, job->gam.as<R>());
   RIX_LAUNCH_CHECK();
   // ring support of every partition's filter on the half plane ju <= N
   {

@@ -63,70 +63,125 @@ constexpr uint32_t kLockPolls = 1u << 22;     // bounded wait for the grid tile'
 static_assert(kTileBytes % 128 == 0, "tile alignment");
 
 // ------------------------------------------------------ partition time -----
-// Per work item: reorder its entries (at most 2048) by first tap, stably
-// (key = tap << 11 | position), the geometry records in place and the sample
-// indices (read from `samples`, in the geometry's current order: the sorted
-// order at partition time, the gridder order when the chunks are rebuilt)
-// into gsamples (which may be `samples`), and flag the entries
-// that start a chunk (the first of a run of one tap, and every limit-th
-// after; limit <= 32, the job's tuning).
-template <typename R>
+// Stable order of the CTA's cnt (<= 2048) entries by tap (< 2^BITS): entry
+// [warp span + 32 r + lane] of a thread is its r-th; dst its place, run its
+// place among the entries of its tap.  A counting sort: ranks within a round of
+// 32 from __match_any_sync, within a warp from its private counts, across warps
+// and taps from scans (a bitonic sort of 2048 keys took 66 barriers; 0.49 ms
+// for the 8.2 M entries of the 1024^2 job).  256 threads.
+template <int BITS>
+struct TapOrder {
+  static constexpr int kBins = 1 << BITS;
+  static constexpr int kRounds = kItemMax / 256;
+  unsigned short cnt[8][kBins];
+  unsigned short off[kBins];
+  int wsum[8];
+
+  // entries per warp
+  static __device__ __forceinline__ int span(int n) { return ((n + 255) / 256) * 32; }
+
+  __device__ __forceinline__ void order(int n, const uint32_t (&tap)[kRounds], int (&dst)[kRounds],
+                                        int (&run)[kRounds]) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int sp = span(n), rounds = sp / 32;
+    for (int i = threadIdx.x; i < 8 * kBins; i += 256) (&cnt[0][0])[i] = 0;
+    __syncthreads();
+    const uint32_t lt = (1u << lane) - 1u;
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r) {
+      if (r < rounds) {
+        const bool valid = warp * sp + 32 * r + lane < n;
+        const uint32_t peers = __match_any_sync(0xffffffffu, valid ? tap[r] : 0x10000u + lane);
+        const int before = valid ? cnt[warp][tap[r]] : 0;
+        run[r] = before + __popc(peers & lt);
+        __syncwarp();
+        if (valid && __ffs(peers) - 1 == lane) cnt[warp][tap[r]] = (unsigned short)(before + __popc(peers));
+        __syncwarp();
+      }
+    }
+    __syncthreads();
+    // per tap: exclusive over the warps; then exclusive over the taps
+    constexpr int PER = kBins / 256;
+    int tot[PER], sum = 0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      const int b = threadIdx.x * PER + k;
+      int acc = 0;
+      for (int w = 0; w < 8; ++w) {
+        const int c = cnt[w][b];
+        cnt[w][b] = (unsigned short)acc;
+        acc += c;
+      }
+      tot[k] = acc;
+      sum += acc;
+    }
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    int base = incl - sum;
+    for (int w = 0; w < warp; ++w) base += wsum[w];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      off[threadIdx.x * PER + k] = (unsigned short)base;
+      base += tot[k];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r)
+      if (r < rounds && warp * sp + 32 * r + lane < n) {
+        run[r] += cnt[warp][tap[r]];
+        dst[r] = off[tap[r]] + run[r];
+      }
+  }
+};
+
+// Per work item: reorder its entries (at most 2048) by first tap, stably, the
+// geometry records in place and the sample indices (read from `samples`, in
+// the geometry's current order: the sorted order at partition time, the
+// gridder order when the chunks are rebuilt) into gsamples (which may be
+// `samples`), and flag the entries that start a chunk (the first of a run of
+// one tap, and every limit-th after).  BITS = 8 for 16 x 16 tiles, 10 for
+// 32 x 32 ones.
+template <typename R, int BITS>
 __global__ void __launch_bounds__(256) k_item_order(const uint32_t* __restrict__ items, int64_t n_items,
                                                     const uint32_t* samples, EntryGeom<R>* geom,
                                                     uint32_t* gsamples, uint32_t* __restrict__ cflag,
                                                     int limit) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  EntryGeom<R>* sg = reinterpret_cast<EntryGeom<R>*>(smem_raw);
-  uint32_t* sk = reinterpret_cast<uint32_t*>(sg + kItemMax);
-  uint32_t* ss = sk + kItemMax;
+  using O = TapOrder<BITS>;
+  __shared__ O sm;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
     const uint32_t e0 = items[item];
     const int cnt = (int)(items[item + 1] - e0);
-    int p2 = 2;
-    while (p2 < cnt) p2 <<= 1;
-    for (int r = threadIdx.x; r < p2; r += blockDim.x) {
-      if (r < cnt) {
-        const EntryGeom<R> g = geom[e0 + r];
-        sg[r] = g;
-        ss[r] = samples[e0 + r];
-        sk[r] = ((g.ouv & 0xffffu) << 11) | (uint32_t)r;
-      } else {
-        sk[r] = 0xffffffffu;
+    const int w0 = warp * O::span(cnt) + lane;
+    const int rounds = O::span(cnt) / 32;
+    EntryGeom<R> g[O::kRounds];
+    uint32_t smp[O::kRounds], tap[O::kRounds];
+    int dst[O::kRounds], run[O::kRounds];
+#pragma unroll
+    for (int r = 0; r < O::kRounds; ++r) {
+      const int i = w0 + 32 * r;
+      tap[r] = 0;
+      if (r < rounds && i < cnt) {
+        g[r] = geom[e0 + i];
+        smp[r] = samples[e0 + i];
+        tap[r] = ((g[r].ouv >> 8) & 0xffu) << (BITS / 2) | (g[r].ouv & 0xffu);
       }
     }
-    __syncthreads();
-    // bitonic sort of sk[0, p2) ascending
-    for (int k = 2; k <= p2; k <<= 1) {
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int i = threadIdx.x; i < p2; i += blockDim.x) {
-          const int ixj = i ^ j;
-          if (ixj > i) {
-            const uint32_t x = sk[i], y = sk[ixj];
-            const bool up = (i & k) == 0;
-            if ((x > y) == up) {
-              sk[i] = y;
-              sk[ixj] = x;
-            }
-          }
-        }
-        __syncthreads();
+    sm.order(cnt, tap, dst, run);   // its barriers separate the reads above from the writes below
+#pragma unroll
+    for (int r = 0; r < O::kRounds; ++r)
+      if (r < rounds && w0 + 32 * r < cnt) {
+        const uint32_t e = e0 + (uint32_t)dst[r];
+        gsamples[e] = smp[r];
+        geom[e] = g[r];
+        cflag[e] = (run[r] % limit) == 0 ? 1u : 0u;
       }
-    }
-    for (int r = threadIdx.x; r < cnt; r += blockDim.x) {
-      const uint32_t key = sk[r];
-      const int src = (int)(key & 2047u);
-      gsamples[e0 + r] = ss[src];
-      geom[e0 + r] = sg[src];
-      // position of the first entry with this tap (lower bound of tap << 11)
-      const uint32_t lo_key = key & ~2047u;
-      int lo = 0, hi = r;
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (sk[mid] < lo_key) lo = mid + 1;
-        else hi = mid;
-      }
-      cflag[e0 + r] = ((r - lo) % limit) == 0 ? 1u : 0u;
-    }
     __syncthreads();
   }
 }
@@ -160,8 +215,7 @@ struct PsfArgs {
   const double* inv_lambda;
   int nchan;
   double scale, half;        // PSF grid coordinate x = u_lambda * scale + half
-  int nw, ww;
-  double w_min, dw;
+  const float4* geom;        // image-grid record per entry (dw, the same on both grids)
   int bt_img, bt, bw;        // key bits per tile coordinate (image grid, PSF window), plane bits
   int win_lo, win_n;         // the partition's PSF window [win_lo, win_lo + win_n)^2
   int64_t e_begin, n;        // the partition's entries
@@ -189,13 +243,7 @@ __global__ void k_psf_geom(PsfArgs a, float4* __restrict__ geom, uint32_t* __res
     const double xs = __dadd_rn(x, -0.5 * kW), ys = __dadd_rn(y, -0.5 * kW);
     const double cx = ceil(xs), cy = ceil(ys);
     int ju = (int)cx - a.win_lo, jv = (int)cy - a.win_lo;
-    float dw = 0.f;
-    if (a.nw > 0) {
-      const double wl = __dmul_rn(a.uvw[row * 3 + 2], sc);
-      const double tw = __ddiv_rn(__dadd_rn(wl, -a.w_min), a.dw);
-      const double pc = fmin(fmax(ceil(tw), 0.0), (double)(a.nw - a.ww));
-      dw = (float)__dadd_rn(pc, -tw);
-    }
+    const float dw = a.geom[e].z;
     // the window holds every footprint of the partition by construction; an
     // entry outside it is flagged (RIX_EINTERNAL) and kept in range
     if (ju < 0 || jv < 0 || ju > a.win_n - kW || jv > a.win_n - kW) {
@@ -256,58 +304,39 @@ __global__ void __launch_bounds__(256) k_psf_order(const uint32_t* __restrict__ 
                                                    const uint32_t* __restrict__ n_items, const float* __restrict__ w,
                                                    float4* geom, float4* __restrict__ ysamp,
                                                    uint32_t* __restrict__ cflag, int limit) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float4* sg = reinterpret_cast<float4*>(smem_raw);
-  uint32_t* sk = reinterpret_cast<uint32_t*>(sg + kItemMax);
-  float* sw = reinterpret_cast<float*>(sk + kItemMax);
+  using O = TapOrder<8>;
+  __shared__ O sm;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t ni = *n_items;
   for (int64_t it = blockIdx.x; it < ni; it += gridDim.x) {
     const uint32_t e0 = items[it];
     const int cnt = (int)(items[it + 1] - e0);
-    int p2 = 2;
-    while (p2 < cnt) p2 <<= 1;
-    for (int r = threadIdx.x; r < p2; r += blockDim.x) {
-      if (r < cnt) {
-        const float4 g = geom[e0 + r];
-        sg[r] = g;
-        sw[r] = w[e0 + r];
-        const uint32_t ouv = __float_as_uint(g.w);
-        sk[r] = ((((ouv >> 8) << 4) | (ouv & 0xffu)) << 11) | (uint32_t)r;   // 8-bit tap, position
-      } else {
-        sk[r] = 0xffffffffu;
+    const int w0 = warp * O::span(cnt) + lane;
+    const int rounds = O::span(cnt) / 32;
+    float4 g[O::kRounds];
+    float wt[O::kRounds];
+    uint32_t tap[O::kRounds];
+    int dst[O::kRounds], run[O::kRounds];
+#pragma unroll
+    for (int r = 0; r < O::kRounds; ++r) {
+      const int i = w0 + 32 * r;
+      tap[r] = 0;
+      if (r < rounds && i < cnt) {
+        g[r] = geom[e0 + i];
+        wt[r] = w[e0 + i];
+        const uint32_t ouv = __float_as_uint(g[r].w);
+        tap[r] = ((ouv >> 8) << 4) | (ouv & 0xffu);
       }
     }
-    __syncthreads();
-    for (int k = 2; k <= p2; k <<= 1) {
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int i = threadIdx.x; i < p2; i += blockDim.x) {
-          const int ixj = i ^ j;
-          if (ixj > i) {
-            const uint32_t x = sk[i], y = sk[ixj];
-            const bool up = (i & k) == 0;
-            if ((x > y) == up) {
-              sk[i] = y;
-              sk[ixj] = x;
-            }
-          }
-        }
-        __syncthreads();
+    sm.order(cnt, tap, dst, run);   // its barriers separate the reads above from the writes below
+#pragma unroll
+    for (int r = 0; r < O::kRounds; ++r)
+      if (r < rounds && w0 + 32 * r < cnt) {
+        const uint32_t e = e0 + (uint32_t)dst[r];
+        geom[e] = g[r];
+        ysamp[e] = make_float4(wt[r], 0.f, wt[r], 0.f);
+        cflag[e] = (run[r] % limit) == 0 ? 1u : 0u;
       }
-    }
-    for (int r = threadIdx.x; r < cnt; r += blockDim.x) {
-      const uint32_t key = sk[r];
-      const int src = (int)(key & 2047u);
-      geom[e0 + r] = sg[src];
-      ysamp[e0 + r] = make_float4(sw[src], 0.f, sw[src], 0.f);
-      const uint32_t lo_key = key & ~2047u;
-      int lo = 0, hi = r;
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (sk[mid] < lo_key) lo = mid + 1;
-        else hi = mid;
-      }
-      cflag[e0 + r] = ((r - lo) % limit) == 0 ? 1u : 0u;
-    }
     __syncthreads();
   }
 }
@@ -1031,10 +1060,7 @@ int launch_psf_fp(const Job* job, int p, double scale, double half, void* planes
     a.nchan = job->desc.nchan;
     a.scale = scale;
     a.half = half;
-    a.nw = job->nw;
-    a.ww = job->ww;
-    a.w_min = job->stats.w_min;
-    a.dw = job->stats.dw;
+    a.geom = job->egeom.as<float4>();
     a.bt_img = job->bt;
     a.bt = bt;
     a.bw = job->bw;
@@ -1064,17 +1090,10 @@ int launch_psf_fp(const Job* job, int p, double scale, double half, void* planes
     ::rix::note_launch();
     k_psf_items<<<eb, 256, 0, st>>>(iflag, iex, n, totals + 1, items);
     if (cudaGetLastError() != cudaSuccess) { rc = set_error(RIX_ECUDA, "PSF work-item launches"); break; }
-    {
-      const size_t sm = (size_t)kItemMax * (sizeof(float4) + 2 * sizeof(uint32_t));
-      if (cudaFuncSetAttribute(k_psf_order, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) {
-        rc = set_error(RIX_ECUDA, "k_psf_order shared memory");
-        break;
-      }
-      ::rix::note_launch();
-      k_psf_order<<<job->ctx->num_sms * 4, 256, sm, st>>>(items, totals + 1, w, geom, ys, f,
-                                                         std::min(std::max(job->chunk_limit, 1), kChunkLimitMax));
-      if (cudaGetLastError() != cudaSuccess) { rc = set_error(RIX_ECUDA, "k_psf_order launch"); break; }
-    }
+    ::rix::note_launch();
+    k_psf_order<<<job->ctx->num_sms * 4, 256, 0, st>>>(items, totals + 1, w, geom, ys, f,
+                                                       std::min(std::max(job->chunk_limit, 1), kChunkLimitMax));
+    if (cudaGetLastError() != cudaSuccess) { rc = set_error(RIX_ECUDA, "k_psf_order launch"); break; }
     if ((rc = scan_exclusive_u32(f, ex, n, totals + 2, st)) != RIX_OK) break;
     ::rix::note_launch();
     k_psf_lists<<<eb, 256, 0, st>>>(f, ex, n, items, totals + 1, totals + 2, chunks, item_chunk);
@@ -1164,21 +1183,16 @@ int grid_work_order(Job* job, cudaStream_t st) {
     rc = set_error(RIX_ENOMEM, "gridder order scratch");
   }
   if (rc == RIX_OK) {
-    const size_t sm = (size_t)kItemMax * (sizeof(EntryGeom<R>) + 2 * sizeof(uint32_t));
-    auto kern = k_item_order<R>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) {
-      rc = set_error(RIX_ECUDA, "k_item_order shared memory");
-    } else {
-      const int blocks = (int)std::min<int64_t>(n_items, (int64_t)job->ctx->num_sms * 4);
-      ::rix::note_launch();
-      // the geometry is in the sorted order right after partitioning, in the
-      // gridder order (with gsamples) when the chunks are rebuilt
-      const uint32_t* in = job->gorder ? job->gsamples.as<uint32_t>() : job->samples.as<uint32_t>();
-      kern<<<blocks, 256, sm, st>>>(job->items.as<uint32_t>(), n_items, in,
-                                    job->egeom.as<EntryGeom<R>>(), job->gsamples.as<uint32_t>(), cflag,
-                                    std::min(std::max(job->chunk_limit, 1), kChunkLimitMax));
-      if (cudaGetLastError() != cudaSuccess) rc = set_error(RIX_ECUDA, "k_item_order launch");
-    }
+    auto kern = job->tile == 16 ? k_item_order<R, 8> : k_item_order<R, 10>;
+    const int blocks = (int)std::min<int64_t>(n_items, (int64_t)job->ctx->num_sms * 4);
+    ::rix::note_launch();
+    // the geometry is in the sorted order right after partitioning, in the
+    // gridder order (with gsamples) when the chunks are rebuilt
+    const uint32_t* in = job->gorder ? job->gsamples.as<uint32_t>() : job->samples.as<uint32_t>();
+    kern<<<blocks, 256, 0, st>>>(job->items.as<uint32_t>(), n_items, in, job->egeom.as<EntryGeom<R>>(),
+                                 job->gsamples.as<uint32_t>(), cflag,
+                                 std::min(std::max(job->chunk_limit, 1), kChunkLimitMax));
+    if (cudaGetLastError() != cudaSuccess) rc = set_error(RIX_ECUDA, "k_item_order launch");
   }
   if (rc == RIX_OK) rc = scan_exclusive_u32(cflag, cidx, n_ent, total, st);
   if (rc == RIX_OK) {
