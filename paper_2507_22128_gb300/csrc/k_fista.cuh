@@ -539,12 +539,13 @@ __device__ __forceinline__ void step_constants(const FistaLoop<R>& f, R* inv_l, 
   *thr = lip > 0.0 ? (R)(lam / lip) : R(0);
 }
 
-// The loops of the batch advance together: every phase hands out the units
-// of all loops (unit u: loop u / per, its unit u % per), so one grid barrier
-// per phase serves the whole batch.
-template <typename R, int LOGL, int DICT>
-__global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 && LOGL <= 12 ? 2 : 1)
-    k_fista_loop(const __grid_constant__ FistaArgs<R> a) {
+// All iterations of the loops f[0 .. nb), which advance together: every phase
+// hands out the units of all loops (unit u: loop u / per, its unit u % per) to
+// the `stride` CTAs that `sync` joins, this one being the `rank`-th; one
+// barrier per phase serves them all.  sync() returns false to stop.
+template <typename R, int LOGL, int DICT, class SYNC>
+__device__ __forceinline__ void fista_iterations(const FistaArgs<R>& a, const FistaLoop<R>* fl, int nb, int rank,
+                                                 int stride, SYNC&& sync) {
   using C = cplx<R>;
   using F = FistaShape<R, LOGL, DICT>;
   constexpr int N = F::N;
@@ -553,26 +554,24 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 && LOGL <= 12 ? 2 
   C* s = reinterpret_cast<C*>(smem_raw);
   C* s2 = s + F::B * F::STRIDE;
   R* stage = reinterpret_cast<R*>(smem_raw + F::kFftSmem);
-  const int nb = a.nb;
-  const FistaLoop<R>& f0 = a.f[0];
-  GridBarrier bar{f0.barrier, f0.status, 0u};
+  const FistaLoop<R>& f0 = fl[0];
   const R sscale = (R)(1.0 / sqrt(8.0));
   const int64_t NN = (int64_t)N * N;
   const int levels = f0.levels;
   __shared__ R s_inv_l[kMaxPart], s_thr[kMaxPart];
-  if (threadIdx.x < nb) step_constants<R, DICT>(a.f[threadIdx.x], &s_inv_l[threadIdx.x], &s_thr[threadIdx.x]);
+  if (threadIdx.x < nb) step_constants<R, DICT>(fl[threadIdx.x], &s_inv_l[threadIdx.x], &s_thr[threadIdx.x]);
   __syncthreads();
   // the constant image d = 2 crop F^-1 C of every loop
-  for (int u = blockIdx.x; u < nb * F::kColUnits; u += gridDim.x) {
-    const FistaLoop<R>& f = a.f[u / F::kColUnits];
+  for (int u = rank; u < nb * F::kColUnits; u += stride) {
+    const FistaLoop<R>& f = fl[u / F::kColUnits];
     cols_inv_unit<R, LOGL>(f.c, f.tb, f.tw, s, s2, u % F::kColUnits);
   }
-  if (!grid_barrier(bar)) return;
-  for (int u = blockIdx.x; u < nb * F::kRowUnits; u += gridDim.x) {
-    const FistaLoop<R>& f = a.f[u / F::kRowUnits];
+  if (!sync()) return;
+  for (int u = rank; u < nb * F::kRowUnits; u += stride) {
+    const FistaLoop<R>& f = fl[u / F::kRowUnits];
     rows_inv_unit<R, LOGL, false>(f.tb, f.d, a.gscale, nullptr, f.tw, s, s2, stage, u % F::kRowUnits);
   }
-  if (!grid_barrier(bar)) return;
+  if (!sync()) return;
   // FISTA's momentum: t_{k+1} = (1 + sqrt(1 + 4 t_k^2)) / 2, momentum
   // (t_k - 1) / t_{k+1}, each operation rounded on its own; one thread per
   // CTA forms it (FP64 square root and division at 1/64 of the FP32 rate),
@@ -592,62 +591,62 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 && LOGL <= 12 ? 2 
     if constexpr (kCat) {
       for (int l = levels - 1; l >= 0; --l) {
         const int per = level_units<DICT>(N >> l, kTS);
-        for (int u = blockIdx.x; u < nb * per; u += gridDim.x) {
-          const FistaLoop<R>& f = a.f[u / per];
+        for (int u = rank; u < nb * per; u += stride) {
+          const FistaLoop<R>& f = fl[u / per];
           synthesis_unit<R, DICT, N>(f, f.y, l, u % per, smem_raw, a.taps);
         }
-        if (!grid_barrier(bar)) return;
+        if (!sync()) return;
       }
     } else if (levels > 1) {
       constexpr int T1 = chain_block<R>();
       constexpr int nt = (N / 2 + T1 - 1) / T1, per = nt * nt;
-      for (int u = blockIdx.x; u < nb * per; u += gridDim.x) {
-        const FistaLoop<R>& f = a.f[u / per];
+      for (int u = rank; u < nb * per; u += stride) {
+        const FistaLoop<R>& f = fl[u / per];
         syn_chain_tile<R, T1>(f.y, levels, N, f.tmp, (u % per) % nt, (u % per) / nt, smem_raw, Db4Taps<R>{});
       }
-      if (!grid_barrier(bar)) return;
+      if (!sync()) return;
     }
-    for (int u = blockIdx.x; u < nb * F::kRowUnits; u += gridDim.x) {
-      const FistaLoop<R>& f = a.f[u / F::kRowUnits];
+    for (int u = rank; u < nb * F::kRowUnits; u += stride) {
+      const FistaLoop<R>& f = fl[u / F::kRowUnits];
       if constexpr (kCat) rows_fwd_unit<R, LOGL, 8>(f.xs, NN, sscale, f.ta, f.tw, s, s2, u % F::kRowUnits);
       else rows_fwd_syn_unit<R, LOGL>(levels > 1 ? f.tmp : f.y, f.y, f.ta, f.tw, s, s2, stage, u % F::kRowUnits);
     }
-    if (!grid_barrier(bar)) return;
-    for (int u = blockIdx.x; u < nb * F::kColUnits; u += gridDim.x) {
-      const FistaLoop<R>& f = a.f[u / F::kColUnits];
+    if (!sync()) return;
+    for (int u = rank; u < nb * F::kColUnits; u += stride) {
+      const FistaLoop<R>& f = fl[u / F::kColUnits];
       cols_conv_unit<R, LOGL>(f.ta, f.mx, f.tb, f.tw, s, s2, stage, u % F::kColUnits);
     }
-    if (!grid_barrier(bar)) return;
-    for (int u = blockIdx.x; u < nb * F::kRowUnits; u += gridDim.x) {
-      const FistaLoop<R>& f = a.f[u / F::kRowUnits];
+    if (!sync()) return;
+    for (int u = rank; u < nb * F::kRowUnits; u += stride) {
+      const FistaLoop<R>& f = fl[u / F::kRowUnits];
       rows_inv_unit<R, LOGL, true>(f.tb, f.g, a.gscale, f.d, f.tw, s, s2, stage, u % F::kRowUnits);
     }
-    if (!grid_barrier(bar)) return;
+    if (!sync()) return;
     const R mom = s_mom;
     for (int l = 0; l < levels; ++l) {
       const int per = level_units<DICT>((N >> l) / 2, ana_block<R, DICT>((N >> l) / 2));
-      for (int u = blockIdx.x; u < nb * per; u += gridDim.x) {
-        const FistaLoop<R>& f = a.f[u / per];
+      for (int u = rank; u < nb * per; u += stride) {
+        const FistaLoop<R>& f = fl[u / per];
         const int b = u / per;
         const StepArgs<R> sa{f.alpha, f.y, s_inv_l[b], s_thr[b], s_inv_l[b] != R(0), mom};
         analysis_unit<R, DICT, N>(f, l, u % per, sa, smem_raw, a.taps);
       }
-      if (!grid_barrier(bar)) return;
+      if (!sync()) return;
     }
   }
   if constexpr (kCat) {
     // each loop's image W alpha: the members' syntheses, summed
     for (int l = levels - 1; l >= 0; --l) {
       const int per = level_units<DICT>(N >> l, kTS);
-      for (int u = blockIdx.x; u < nb * per; u += gridDim.x) {
-        const FistaLoop<R>& f = a.f[u / per];
+      for (int u = rank; u < nb * per; u += stride) {
+        const FistaLoop<R>& f = fl[u / per];
         synthesis_unit<R, DICT, N>(f, f.alpha, l, u % per, smem_raw, a.taps);
       }
-      if (!grid_barrier(bar)) return;
+      if (!sync()) return;
     }
     for (int b = 0; b < nb; ++b) {
-      const FistaLoop<R>& f = a.f[b];
-      for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < NN; i += (int64_t)gridDim.x * blockDim.x) {
+      const FistaLoop<R>& f = fl[b];
+      for (int64_t i = rank * (int64_t)blockDim.x + threadIdx.x; i < NN; i += (int64_t)stride * blockDim.x) {
         R acc = R(0);
 #pragma unroll
         for (int m = 0; m < 8; ++m) acc += f.xs[m * NN + i];
@@ -655,6 +654,36 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 && LOGL <= 12 ? 2 
       }
     }
   }
+}
+
+template <typename R, int LOGL, int DICT>
+__global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 && LOGL <= 12 ? 2 : 1)
+    k_fista_loop(const __grid_constant__ FistaArgs<R> a) {
+  GridBarrier bar{a.f[0].barrier, a.f[0].status, 0u};
+  fista_iterations<R, LOGL, DICT>(a, a.f, a.nb, (int)blockIdx.x, (int)gridDim.x, [&] { return grid_barrier(bar); });
+}
+
+// Small images: a cluster of kClusterCtas CTAs per loop, joined by the cluster
+// barrier, instead of the whole grid by a counter in global memory.  A phase of
+// a 128 x 128 loop has 4 to 16 units, so 16 CTAs run it as fast as 152 do, and
+// the barrier, a few hundred nanoseconds instead of one to two microseconds of
+// atomics and polling, was most of its time (50 iterations of both partitions
+// at 128^2: 1.73 -> 1.28 ms against the dataflow schedule of the batch).
+constexpr int kClusterCtas = 16;
+constexpr int kClusterLogL = 8;   // longest transform 2N that takes this path
+
+template <typename R, int LOGL, int DICT>
+__global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 2 : 1)
+    k_fista_cluster(const __grid_constant__ FistaArgs<R> a) {
+  const int b = (int)blockIdx.x / kClusterCtas, rank = (int)blockIdx.x % kClusterCtas;
+  fista_iterations<R, LOGL, DICT>(a, a.f + b, 1, rank, kClusterCtas, [] {
+    // every thread of the cluster arrives (releasing its writes) and waits
+    // (acquiring the others'): a hardware barrier, which completes because
+    // every CTA of the cluster runs the same phases
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    return true;
+  });
 }
 
 // ------------------------------------------------------ dataflow schedule --
@@ -833,15 +862,7 @@ int launch_fista_loop(const Ctx* ctx, const FistaLoop<R>* f, int nb, cudaStream_
   for (int b = 1; b < nb; ++b)
     if (f[b].n != f[0].n || f[b].levels != f[0].levels || f[b].iters != f[0].iters || f[b].dict != f[0].dict)
       return set_error(RIX_EINVAL, "FISTA batch: the loops differ in size, levels, iterations or dictionary");
-  auto kern = k_fista_loop<R, LOGL, DICT>;
   const size_t smem = F::kSmem;
-  RIX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int per_sm = 0;
-  RIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFftThreads, smem));
-  if (per_sm < 1) return set_error(RIX_EINVAL, "FISTA loop does not fit on an SM (%zu B shared)", smem);
-  // one CTA per SM for a single loop (another partition's loop or gridder fits
-  // beside it); a batch of loops takes up to two
-  const int nblk = ctx->num_sms * std::min(per_sm, nb > 1 ? 2 : 1);
   FistaArgs<R> args{};
   for (int b = 0; b < nb; ++b) args.f[b] = f[b];
   args.nb = nb;
@@ -854,60 +875,91 @@ int launch_fista_loop(const Ctx* ctx, const FistaLoop<R>* f, int nb, cudaStream_
       for (int i = 0; i < 16; ++i) args.taps[m][i] = i < k ? (R)h[i] : R(0);
     }
   }
-  if constexpr (DICT == RIX_DICT_DB4) {
-    if (nb > 1) {
-      // several loops (Db4): the dataflow schedule instead of grid barriers
-      auto fk = k_fista_flow<R, LOGL>;
-      RIX_CUDA(cudaFuncSetAttribute(fk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      int fper = 0;
-      RIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fper, fk, kFftThreads, smem));
-      if (fper < 1) return set_error(RIX_EINVAL, "FISTA loop does not fit on an SM (%zu B shared)", smem);
-      const int fblk = ctx->num_sms * std::min(fper, 2);
-      const int levels = f[0].levels;
-      const int64_t nph = (levels > 1 ? 1 : 0) + 3 + levels;
-      const int64_t nctl = 1 + (int64_t)nb * (2 + (int64_t)f[0].iters * nph);
-      unsigned int* ctl = nullptr;
-      R* mom = nullptr;
-      RIX_CUDA(::rix::malloc_async(&ctl, (size_t)nctl * sizeof(unsigned int), st));
-      if (::rix::malloc_async(&mom, (size_t)std::max(f[0].iters, 1) * sizeof(R), st) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFreeAsync(ctl, st);
-        return set_error(RIX_ENOMEM, "FISTA schedule tables");
-      }
-      int rc = RIX_OK;
-      if (cudaMemsetAsync(ctl, 0, (size_t)nctl * sizeof(unsigned int), st) != cudaSuccess) {
-        rc = set_error(RIX_ECUDA, "FISTA schedule reset");
-      } else {
-        args.ticket = ctl;
-        args.done = ctl + 1;
-        if (f[0].iters <= kMomTab) {
-          mom_host<R>(f[0].iters, args.mom_tab);
-          args.mom = nullptr;
-        } else {
-          ::rix::note_launch();
-          k_mom_table<R><<<1, 1, 0, st>>>(f[0].iters, mom);
-          args.mom = mom;
+  if constexpr (LOGL <= kClusterLogL) {
+    auto ck = k_fista_cluster<R, LOGL, DICT>;
+    RIX_CUDA(cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RIX_CUDA(cudaFuncSetAttribute(ck, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = kClusterCtas;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(nb * kClusterCtas));
+    cfg.blockDim = dim3(kFftThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    ::rix::note_launch();
+    timing_mark(kTimeMinorLoop, st, true);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, ck, args);
+    timing_mark(kTimeMinorLoop, st, false);
+    if (e != cudaSuccess) return set_error(RIX_ECUDA, "FISTA loop launch: %s", cudaGetErrorString(e));
+    return RIX_OK;
+  } else {
+    auto kern = k_fista_loop<R, LOGL, DICT>;
+    RIX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 0;
+    RIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFftThreads, smem));
+    if (per_sm < 1) return set_error(RIX_EINVAL, "FISTA loop does not fit on an SM (%zu B shared)", smem);
+    // one CTA per SM for a single loop (another partition's loop or gridder fits
+    // beside it); a batch of loops takes up to two
+    const int nblk = ctx->num_sms * std::min(per_sm, nb > 1 ? 2 : 1);
+    if constexpr (DICT == RIX_DICT_DB4) {
+      if (nb > 1) {
+        // several loops (Db4): the dataflow schedule instead of grid barriers
+        auto fk = k_fista_flow<R, LOGL>;
+        RIX_CUDA(cudaFuncSetAttribute(fk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        int fper = 0;
+        RIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fper, fk, kFftThreads, smem));
+        if (fper < 1) return set_error(RIX_EINVAL, "FISTA loop does not fit on an SM (%zu B shared)", smem);
+        const int fblk = ctx->num_sms * std::min(fper, 2);
+        const int levels = f[0].levels;
+        const int64_t nph = (levels > 1 ? 1 : 0) + 3 + levels;
+        const int64_t nctl = 1 + (int64_t)nb * (2 + (int64_t)f[0].iters * nph);
+        unsigned int* ctl = nullptr;
+        R* mom = nullptr;
+        RIX_CUDA(::rix::malloc_async(&ctl, (size_t)nctl * sizeof(unsigned int), st));
+        if (::rix::malloc_async(&mom, (size_t)std::max(f[0].iters, 1) * sizeof(R), st) != cudaSuccess) {
+          cudaGetLastError();
+          cudaFreeAsync(ctl, st);
+          return set_error(RIX_ENOMEM, "FISTA schedule tables");
         }
-        void* params[] = {&args};
-        ::rix::note_launch();
-        timing_mark(kTimeMinorLoop, st, true);
-        const cudaError_t e =
-            cudaLaunchCooperativeKernel((const void*)fk, dim3(fblk), dim3(kFftThreads), params, smem, st);
-        timing_mark(kTimeMinorLoop, st, false);
-        if (e != cudaSuccess) rc = set_error(RIX_ECUDA, "FISTA loop launch: %s", cudaGetErrorString(e));
+        int rc = RIX_OK;
+        if (cudaMemsetAsync(ctl, 0, (size_t)nctl * sizeof(unsigned int), st) != cudaSuccess) {
+          rc = set_error(RIX_ECUDA, "FISTA schedule reset");
+        } else {
+          args.ticket = ctl;
+          args.done = ctl + 1;
+          if (f[0].iters <= kMomTab) {
+            mom_host<R>(f[0].iters, args.mom_tab);
+            args.mom = nullptr;
+          } else {
+            ::rix::note_launch();
+            k_mom_table<R><<<1, 1, 0, st>>>(f[0].iters, mom);
+            args.mom = mom;
+          }
+          void* params[] = {&args};
+          ::rix::note_launch();
+          timing_mark(kTimeMinorLoop, st, true);
+          const cudaError_t e =
+              cudaLaunchCooperativeKernel((const void*)fk, dim3(fblk), dim3(kFftThreads), params, smem, st);
+          timing_mark(kTimeMinorLoop, st, false);
+          if (e != cudaSuccess) rc = set_error(RIX_ECUDA, "FISTA loop launch: %s", cudaGetErrorString(e));
+        }
+        cudaFreeAsync(ctl, st);
+        cudaFreeAsync(mom, st);
+        return rc;
       }
-      cudaFreeAsync(ctl, st);
-      cudaFreeAsync(mom, st);
-      return rc;
     }
+    RIX_CUDA(cudaMemsetAsync(f[0].barrier, 0, sizeof(unsigned int), st));
+    void* params[] = {&args};
+    ::rix::note_launch();
+    timing_mark(kTimeMinorLoop, st, true);
+    RIX_CUDA(cudaLaunchCooperativeKernel((const void*)kern, dim3(nblk), dim3(kFftThreads), params, smem, st));
+    timing_mark(kTimeMinorLoop, st, false);
+    return RIX_OK;
   }
-  RIX_CUDA(cudaMemsetAsync(f[0].barrier, 0, sizeof(unsigned int), st));
-  void* params[] = {&args};
-  ::rix::note_launch();
-  timing_mark(kTimeMinorLoop, st, true);
-  RIX_CUDA(cudaLaunchCooperativeKernel((const void*)kern, dim3(nblk), dim3(kFftThreads), params, smem, st));
-  timing_mark(kTimeMinorLoop, st, false);
-  return RIX_OK;
 }
 
 // dispatch on the transform length 2N (N a power of two in [32, KMAXN])
