@@ -291,17 +291,45 @@ int idwt2(const Ctx* ctx, const R* c, R* out, R* tmp, int N, int levels, cudaStr
 namespace {
 
 // --------------------------------------------------------------- ms-CLEAN ----
-template <typename R>
-struct Cand {
-  R val;       // b_s |R_s(p)| / P_ss(0); -1 = none
-  R rval;      // R_s(p), signed
-  int s, pix;
-  R r0max;     // max |R_0| over the image
+// Candidate values are compared as integers: the bit pattern of a float, with
+// the lower bits flipped where the sign is set, orders as the value does.  FP64
+// comparisons run at 1/64 of the FP32 rate, and the reductions' alone took a
+// third of an FP64 iteration (25 us at 512^2 with three scales).
+template <typename R> struct OrdKey;
+template <> struct OrdKey<float> {
+  using K = int;
+  static constexpr K kInf = 0x7f800000;
+  static __device__ __forceinline__ K of(float v) { const K b = __float_as_int(v); return b ^ ((b >> 31) & 0x7fffffff); }
+  static __device__ __forceinline__ float value(K k) { return __int_as_float(k ^ ((k >> 31) & 0x7fffffff)); }
+  static __device__ __forceinline__ K of_abs(float v) { return __float_as_int(v) & 0x7fffffff; }
+};
+template <> struct OrdKey<double> {
+  using K = long long;
+  static constexpr K kInf = 0x7ff0000000000000ll;
+  static __device__ __forceinline__ K of(double v) {
+    const K b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+  }
+  static __device__ __forceinline__ double value(K k) { return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll)); }
+  static __device__ __forceinline__ K of_abs(double v) { return __double_as_longlong(v) & 0x7fffffffffffffffll; }
 };
 
 template <typename R>
+struct Cand {
+  typename OrdKey<R>::K key;   // of b_s |R_s(p)| / P_ss(0); of -1 = none
+  R rval;                      // R_s(p), signed
+  int s, pix;
+  typename OrdKey<R>::K r0max; // of max |R_0| over the image
+};
+
+template <typename R>
+__device__ __forceinline__ Cand<R> no_cand() {
+  return Cand<R>{OrdKey<R>::of(R(-1)), R(0), 0x7fffffff, 0x7fffffff, 0};
+}
+
+template <typename R>
 __device__ __forceinline__ bool better(const Cand<R>& a, const Cand<R>& b) {
-  if (a.val != b.val) return a.val > b.val;
+  if (a.key != b.key) return a.key > b.key;
   if (a.s != b.s) return a.s < b.s;
   return a.pix < b.pix;
 }
@@ -309,7 +337,7 @@ __device__ __forceinline__ bool better(const Cand<R>& a, const Cand<R>& b) {
 template <typename R>
 __device__ __forceinline__ Cand<R> shfl_cand(const Cand<R>& c, int o) {
   Cand<R> r;
-  r.val = __shfl_xor_sync(0xffffffffu, c.val, o);
+  r.key = __shfl_xor_sync(0xffffffffu, c.key, o);
   r.rval = __shfl_xor_sync(0xffffffffu, c.rval, o);
   r.s = __shfl_xor_sync(0xffffffffu, c.s, o);
   r.pix = __shfl_xor_sync(0xffffffffu, c.pix, o);
@@ -320,7 +348,7 @@ __device__ __forceinline__ Cand<R> shfl_cand(const Cand<R>& c, int o) {
 template <typename R>
 __device__ __forceinline__ Cand<R> merge(const Cand<R>& a, const Cand<R>& b) {
   Cand<R> r = better(b, a) ? b : a;
-  r.r0max = fmax(a.r0max, b.r0max);
+  r.r0max = a.r0max > b.r0max ? a.r0max : b.r0max;
   return r;
 }
 
@@ -333,7 +361,7 @@ __device__ Cand<R> block_reduce(Cand<R> c, Cand<R>* sh) {
   if (lane == 0) sh[warp] = c;
   __syncthreads();
   if (warp == 0) {
-    Cand<R> d = lane < nw ? sh[lane] : Cand<R>{R(-1), R(0), 0x7fffffff, 0x7fffffff, R(0)};
+    Cand<R> d = lane < nw ? sh[lane] : no_cand<R>();
     for (int o = 16; o; o >>= 1) d = merge(d, shfl_cand(d, o));
     if (lane == 0) sh[0] = d;
   }
@@ -351,7 +379,8 @@ struct CleanArgs {
   void* model;                 // [n][n]
   const void* stencil;         // concatenated (2r+1)^2 stencils of B_s
   int st_off[kMaxScales], st_rad[kMaxScales];
-  void* slots;                 // Cand<R> [2][gridDim]
+  const float2* reach;         // k_clean_reach's table
+  void* slots;                 // Slot<R> [2][gridDim]
   int* comp_s;                 // [niter]
   int* comp_pix;
   double* comp_amp;
@@ -360,85 +389,249 @@ struct CleanArgs {
   int* status;                 // the job's status word
 };
 
-// The whole minor cycle in one cooperative launch: each iteration subtracts
-// the previous component from every scale residual and, in the same sweep,
-// finds the next peak; one bounded grid barrier per iteration separates the
-// sweep from the global reduction (double-buffered candidate slots).  A
-// barrier that gives up (RIX_ETIMEOUT in the status word) ends every CTA.
-// NS = the number of scales, fixed at compile time so that a sweep issues
-// the loads of every scale of a pixel together.
-template <typename R, int NS>
+// candidate value b_s |R_s| / P_ss(0) as |R_s| times b_s / P_ss(0) (a scale
+// whose peak is 0 never wins: 0; the loop stops if it is chosen)
+template <typename R>
+__device__ __forceinline__ R clean_scale(const CleanArgs& a, R peak, int s) {
+  return peak != R(0) ? (R)a.bias[s] / peak : R(0);
+}
+
+// How far a component of scale sc moves the candidates of a TS x TS block of
+// the (2n)^2 grid of relative positions, per unit amplitude: x = the largest
+// |P_{s,sc}| b_s / P_ss(0) over the allowed scales, y = the largest |P_{0,sc}|
+// (rounded up; infinite where a value is not finite), [ns][2n / TS][2n / TS].
+// One warp per block.
+template <typename R, int TS>
+__global__ void __launch_bounds__(256) k_clean_reach(CleanArgs a, float2* __restrict__ out) {
+  const int n2 = 2 * a.n, nb = n2 / TS, ns = a.ns;
+  const int64_t n2sq = (int64_t)n2 * n2, blocks = (int64_t)ns * nb * nb;
+  const R* P = static_cast<const R*>(a.P);
+  const int lane = threadIdx.x & 31;
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < blocks;
+       i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const int sc = (int)(i / ((int64_t)nb * nb));
+    const int rem = (int)(i - (int64_t)sc * nb * nb), by = rem / nb, bx = rem - by * nb;
+    float gx = 0.f, gy = 0.f;
+    for (int s = 0; s < ns; ++s) {
+      if (s > 0 && !((a.allowed >> s) & 1)) continue;
+      const R* p = P + (int64_t)(s * ns + sc) * n2sq + (int64_t)by * TS * n2 + bx * TS;
+      R m = R(0);
+      bool fin = true;
+      for (int k = lane; k < TS * TS; k += 32) {
+        const R v = fabs(p[(int64_t)(k / TS) * n2 + k % TS]);
+        fin = fin && v <= (sizeof(R) == 4 ? R(3.4e38) : R(1e300));
+        m = m > v ? m : v;
+      }
+      const float mf = fin ? (float)m * 1.00001f + 1e-37f : __int_as_float(0x7f800000);
+      const R pk = P[((int64_t)(s * ns + s) * n2 + a.n) * n2 + a.n];
+      if ((a.allowed >> s) & 1) gx = fmaxf(gx, mf * (fabsf((float)clean_scale<R>(a, pk, s)) * 1.00001f));
+      if (s == 0) gy = mf;
+    }
+    for (int o = 16; o; o >>= 1) {
+      gx = fmaxf(gx, __shfl_xor_sync(0xffffffffu, gx, o));
+      gy = fmaxf(gy, __shfl_xor_sync(0xffffffffu, gy, o));
+    }
+    if (lane == 0) out[i] = make_float2(gx, gy);
+  }
+}
+
+// what a CTA hands the others at an iteration: its best candidate, and the
+// value and pixel of the second best CTA once slots are merged
+template <typename R>
+struct Slot {
+  Cand<R> c;
+  typename OrdKey<R>::K key2;
+  int pix2;
+};
+template <typename R>
+__device__ __forceinline__ Slot<R> merge(const Slot<R>& a, const Slot<R>& b) {
+  const bool bw = better(b.c, a.c);
+  Slot<R> r;
+  r.c = merge(a.c, b.c);
+  const typename OrdKey<R>::K lk = bw ? a.c.key : b.c.key, wk = bw ? b.key2 : a.key2;
+  const int lp = bw ? a.c.pix : b.c.pix, wp = bw ? b.pix2 : a.pix2;
+  r.key2 = lk > wk ? lk : wk;
+  r.pix2 = lk > wk ? lp : wp;
+  return r;
+}
+template <typename R>
+__device__ __forceinline__ Slot<R> shfl_slot(const Slot<R>& s, int o) {
+  Slot<R> r;
+  r.c = shfl_cand(s.c, o);
+  r.key2 = __shfl_xor_sync(0xffffffffu, s.key2, o);
+  r.pix2 = __shfl_xor_sync(0xffffffffu, s.pix2, o);
+  return r;
+}
+template <typename R>
+__device__ __forceinline__ Slot<R> no_slot() {
+  return Slot<R>{no_cand<R>(), OrdKey<R>::of(R(-1)), 0};
+}
+
+// A CTA's own TS x TS tiles of the image.
+template <typename R>
+struct CleanTile {
+  Cand<R> c;        // exact after the first `upto` components
+  int upto;
+  float val, r0;    // c's value and r0max, rounded up
+  float grow, grow0;   // bounds of their change by the later components
+};
+
+constexpr int kCleanSweep = 16;   // iterations between two updates of every tile
+
+// The whole minor cycle in one cooperative launch.  The components are those
+// of updating every scale residual at every iteration, and every residual
+// value goes through the same subtractions in the same order, but a tile is
+// updated only when it could hold the next peak: its last exact maximum plus
+// the reach of the components since (k_clean_reach) is compared with a lower
+// bound of the next peak, the larger of the cleaned peak's remainder and the
+// runner-up's value less the new component's reach there.  All tiles catch up
+// every kCleanSweep iterations, so the work stays even and the residuals are
+// read and written once per sweep instead of once per component: at 2048^2
+// with four scales 43 -> 26 us per iteration (201 MB moved by each before), at
+// 512^2 in FP64 with three 25 -> 15 us (the integer comparisons included).  The stopping rule needs max |R_0| < threshold exactly: a CTA none
+// of whose tiles is surely above it updates those that could be.
+// One bounded grid barrier per iteration separates the updates from the
+// selection (double-buffered slots); a barrier that gives up (RIX_ETIMEOUT in
+// the status word) ends every CTA.  NS = the number of scales.
+template <typename R, int NS, int TS>
 __global__ void __launch_bounds__(256) k_msclean(CleanArgs a) {
+  using Key = OrdKey<R>;
+  constexpr int PX = TS * TS / 256;
   GridBarrier bar{a.barrier, a.status, 0u};
   __shared__ Cand<R> sh[32];
-  const int n = a.n, n2 = 2 * a.n;
-  const int64_t npix = (int64_t)n * n;
+  __shared__ Slot<R> shs[8];
+  __shared__ int s_need0;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  CleanTile<R>* tile = reinterpret_cast<CleanTile<R>*>(smem_raw);
+  const int n = a.n, n2 = 2 * a.n, nt = n / TS, nb = n2 / TS;
+  const int ntiles = nt * nt;
+  const int ntl = (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // tiles blockIdx + i gridDim
+  int* hot = reinterpret_cast<int*>(tile + (ntiles + gridDim.x - 1) / gridDim.x);
+  const int64_t npix = (int64_t)n * n, n2sq = (int64_t)n2 * n2;
   R* __restrict__ Rs = static_cast<R*>(a.R);
   const R* __restrict__ P = static_cast<const R*>(a.P);
-  Cand<R>* slots = static_cast<Cand<R>*>(a.slots);
+  Slot<R>* slots = static_cast<Slot<R>*>(a.slots);
   __shared__ R peak[kMaxScales], scl[kMaxScales];
   if (threadIdx.x < NS) {
     const int s = threadIdx.x;
     peak[s] = P[((int64_t)(s * NS + s) * n2 + n) * n2 + n];
-    // the candidate value b_s |R_s| / P_ss(0) as |R_s| times b_s / P_ss(0)
-    // (a scale whose peak is 0 never wins: 0; the loop stops if it is chosen)
-    scl[s] = peak[s] != R(0) ? (R)a.bias[s] / peak[s] : R(0);
+    scl[s] = clean_scale<R>(a, peak[s], s);
   }
   __syncthreads();
-  const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
-  const int logn = 31 - __clz(n);   // n is a power of two
-  const int64_t n2sq = (int64_t)n2 * n2;
 
-  // sweep with the subtraction of component (sc, py, px, amp) (amp = 0: none)
-  auto sweep = [&](int sc, int py, int px, R amp) {
-    Cand<R> c{R(-1), R(0), 0x7fffffff, 0x7fffffff, R(0)};
-    const R* __restrict__ psc = P + (int64_t)sc * n2sq;   // P_{s, sc} = psc + s NS (2n)^2
-    for (int64_t i = gtid; i < npix; i += gstride) {
-      const int y = (int)(i >> logn), x = (int)(i & (n - 1));
+  // brings tile i up to `upto` components (the last one given, the others read
+  // back) and finds its candidate
+  auto update = [&](int i, int upto, int sl, int pl, R al) {
+    const int t = (int)blockIdx.x + i * (int)gridDim.x;
+    const int y0 = (t / nt) * TS + (int)threadIdx.x / TS, x = (t % nt) * TS + (int)threadIdx.x % TS;
+    constexpr int DY = 256 / TS;
+    R v[PX][NS];
+#pragma unroll
+    for (int k = 0; k < PX; ++k)
+#pragma unroll
+      for (int s = 0; s < NS; ++s) v[k][s] = Rs[s * npix + (int64_t)(y0 + k * DY) * n + x];
+    const int from = tile[i].upto;
+#pragma unroll 2
+    for (int c = from; c < upto; ++c) {
+      const bool own = c == upto - 1;
+      const int sc = own ? sl : __ldcg(a.comp_s + c), pix = own ? pl : __ldcg(a.comp_pix + c);
+      const R amp = own ? al : (R)__ldcg(a.comp_amp + c);
+      const int py = pix / n, px = pix - py * n;
       // P_{s,sc}(y - py, x - px) on the centred 2n grid
-      const int64_t pp = (int64_t)(n + y - py) * n2 + (n + x - px);
-      R v[NS];
+      const R* __restrict__ q = P + (int64_t)sc * n2sq + (int64_t)(n + y0 - py) * n2 + (n + x - px);
+      R w[PX][NS];
 #pragma unroll
-      for (int s = 0; s < NS; ++s) v[s] = Rs[s * npix + i];
+      for (int k = 0; k < PX; ++k)
+#pragma unroll
+        for (int s = 0; s < NS; ++s) w[k][s] = q[(int64_t)s * NS * n2sq + (int64_t)k * DY * n2];
       if (amp != R(0)) {
-        R q[NS];
 #pragma unroll
-        for (int s = 0; s < NS; ++s) q[s] = psc[(int64_t)s * NS * n2sq + pp];
+        for (int k = 0; k < PX; ++k)
 #pragma unroll
-        for (int s = 0; s < NS; ++s) {
-          v[s] -= amp * q[s];
-          Rs[s * npix + i] = v[s];
-        }
+          for (int s = 0; s < NS; ++s) v[k][s] -= amp * w[k][s];
       }
+    }
+    Cand<R> c = no_cand<R>();
+#pragma unroll
+    for (int k = 0; k < PX; ++k) {
+      const int pix = (y0 + k * DY) * n + x;
 #pragma unroll
       for (int s = 0; s < NS; ++s) {
-        const R av = fabs(v[s]);
-        if (s == 0) c.r0max = fmax(c.r0max, av);
+        if (upto > from) Rs[s * npix + pix] = v[k][s];
+        // (a NaN is no candidate and no maximum)
+        const typename Key::K ak = Key::of_abs(v[k][s]);
+        if (s == 0 && ak > c.r0max && ak <= Key::kInf) c.r0max = ak;
         if ((a.allowed >> s) & 1) {
-          const R val = av * scl[s];
-          if (val > c.val || (val == c.val && (s < c.s || (s == c.s && (int)i < c.pix)))) {
-            c.val = val;
-            c.rval = v[s];
+          const typename Key::K key = Key::of(fabs(v[k][s]) * scl[s]);
+          if (key >= c.key && key <= Key::kInf && (key > c.key || s < c.s || (s == c.s && pix < c.pix))) {
+            c.key = key;
+            c.rval = v[k][s];
             c.s = s;
-            c.pix = (int)i;
+            c.pix = pix;
           }
         }
       }
     }
-    return block_reduce(c, sh);
+    c = block_reduce(c, sh);
+    if (threadIdx.x == 0) {
+      CleanTile<R>& e = tile[i];
+      e.c = c;
+      e.upto = upto;
+      e.val = (float)Key::value(c.key) * 1.00001f;
+      e.r0 = (float)Key::value(c.r0max) * 1.00001f;
+      e.grow = e.grow0 = 0.f;
+    }
+  };
+  // the CTA's slot after `upto` components: its best exact candidate, and a
+  // value of |R_0| that its tiles reach
+  auto publish = [&](int upto) {
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      Cand<R> c = no_cand<R>();
+      for (int i = threadIdx.x; i < ntl; i += 32) {
+        Cand<R> e = tile[i].c;
+        if (tile[i].upto != upto) {
+          const float low = tile[i].r0 * 0.9999f - tile[i].grow0;
+          e = no_cand<R>();
+          e.r0max = low > 0.f ? Key::of((R)low) : 0;
+        }
+        c = merge(c, e);
+      }
+      for (int o = 16; o; o >>= 1) c = merge(c, shfl_cand(c, o));
+      if (threadIdx.x == 0) slots[(int64_t)(upto & 1) * gridDim.x + blockIdx.x] = Slot<R>{c, Key::of(R(-1)), 0};
+    }
+  };
+  // the reach of a component at `pix` over the TS x TS square at (y0, x0)
+  auto reach = [&](int sc, int y0, int x0, int pix) -> float2 {
+    const int py = pix / n, px = pix - py * n;
+    const int ya = (n + y0 - py) / TS, yb = (n + y0 + TS - 1 - py) / TS;
+    const int xa = (n + x0 - px) / TS, xb = (n + x0 + TS - 1 - px) / TS;
+    const float2* g = a.reach + (int64_t)sc * nb * nb;
+    const float2 e = g[(int64_t)ya * nb + xa], f = g[(int64_t)ya * nb + xb];
+    const float2 h = g[(int64_t)yb * nb + xa], k = g[(int64_t)yb * nb + xb];
+    return make_float2(fmaxf(fmaxf(e.x, f.x), fmaxf(h.x, k.x)), fmaxf(fmaxf(e.y, f.y), fmaxf(h.y, k.y)));
   };
 
-  Cand<R> loc = sweep(0, 0, 0, R(0));
-  if (threadIdx.x == 0) slots[blockIdx.x] = loc;
+  for (int i = threadIdx.x; i < ntl; i += 256) tile[i].upto = 0;
+  __syncthreads();
+  for (int i = 0; i < ntl; ++i) update(i, 0, 0, 0, R(0));
+  publish(0);
+  const float thr = (float)a.threshold;
   int it = 0;
   for (;; ++it) {
     if (!grid_barrier(bar)) return;
-    const Cand<R>* cur = slots + (int64_t)(it & 1) * gridDim.x;
-    Cand<R> c{R(-1), R(0), 0x7fffffff, 0x7fffffff, R(0)};
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) c = merge(c, cur[b]);
-    const Cand<R> best = block_reduce(c, sh);
-    if (it >= a.niter || best.r0max < (R)a.threshold || best.val < R(0) || peak[best.s] == R(0)) break;
+    const Slot<R>* cur = slots + (int64_t)(it & 1) * gridDim.x;
+    Slot<R> b = no_slot<R>();
+    for (int k = threadIdx.x; k < (int)gridDim.x; k += 256) b = merge(b, cur[k]);
+    for (int o = 16; o; o >>= 1) b = merge(b, shfl_slot(b, o));
+    if ((threadIdx.x & 31) == 0) shs[threadIdx.x >> 5] = b;
+    if (threadIdx.x == 0) s_need0 = 0;
+    __syncthreads();
+    b = shs[0];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) b = merge(b, shs[k]);
+    const Cand<R> best = b.c;
+    if (it >= a.niter || Key::value(best.r0max) < (R)a.threshold || best.key < 0 || peak[best.s] == R(0)) break;
     const R amp = (R)a.gain * best.rval / peak[best.s];
     const int py = best.pix / n, px = best.pix - py * n;
     if (blockIdx.x == 0) {
@@ -457,8 +650,32 @@ __global__ void __launch_bounds__(256) k_msclean(CleanArgs a) {
         if (yy >= 0 && yy < n && xx >= 0 && xx < n) model[(int64_t)yy * n + xx] += amp * stn[k];
       }
     }
-    loc = sweep(best.s, py, px, amp);
-    if (threadIdx.x == 0) slots[(int64_t)((it + 1) & 1) * gridDim.x + blockIdx.x] = loc;
+    // a lower bound of the next peak
+    const float fa = fabsf((float)amp) * 1.00001f;
+    const float keep = (float)Key::value(best.key) * (1.f - (float)a.gain) * 0.9999f;
+    float low = keep;
+    if (b.key2 > 0) {
+      const int y2 = b.pix2 / n, x2 = b.pix2 - (b.pix2 / n) * n;
+      const float v2 = (float)Key::value(b.key2) * 0.9999f - fa * reach(best.s, (y2 / TS) * TS, (x2 / TS) * TS, best.pix).x;
+      low = fmaxf(low, v2);
+    }
+    const bool all = (it + 1) % kCleanSweep == 0;
+    for (int i = threadIdx.x; i < ntl; i += 256) {
+      CleanTile<R>& e = tile[i];
+      const int t = (int)blockIdx.x + i * (int)gridDim.x;
+      const float2 g = reach(best.s, (t / nt) * TS, (t % nt) * TS, best.pix);
+      e.grow += fa * g.x;
+      e.grow0 += fa * g.y;
+      // (written so that a value that is not a number updates the tile)
+      hot[i] = all || !((e.val + e.grow) * 1.0001f < low);
+      if (a.threshold > 0.0 && e.r0 * 0.9999f - e.grow0 >= thr * 1.0001f) s_need0 = 1;   // surely above
+    }
+    __syncthreads();
+    const bool above = a.threshold <= 0.0 || s_need0 != 0;
+    for (int i = 0; i < ntl; ++i)
+      if (hot[i] || (!above && !((tile[i].r0 + tile[i].grow0) * 1.0001f < thr * 0.9999f)))
+        update(i, it + 1, best.s, best.pix, amp);
+    publish(it + 1);
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) *a.count = it;
 }
@@ -803,27 +1020,34 @@ int op_msclean(Job* job, int p, const rix_msclean_params* prm, R* delta_out, cud
   }
   // state: delta image, components, slots
   const int cap = std::max(prm->niter, 1);
-  int per_sm = 0;
+  // 32 x 32 tiles, 16 x 16 for small images (a tile per CTA down to 64^2)
+  const int ts = n >= 512 ? 32 : 16;
   void (*kern)(CleanArgs) = nullptr;
+#define RIX_CLEAN(NS) \
+  case NS: kern = ts == 32 ? k_msclean<R, NS, 32> : k_msclean<R, NS, 16>; break;
   switch (ns) {
-    case 1: kern = k_msclean<R, 1>; break;
-    case 2: kern = k_msclean<R, 2>; break;
-    case 3: kern = k_msclean<R, 3>; break;
-    case 4: kern = k_msclean<R, 4>; break;
-    case 5: kern = k_msclean<R, 5>; break;
-    case 6: kern = k_msclean<R, 6>; break;
-    case 7: kern = k_msclean<R, 7>; break;
-    case 8: kern = k_msclean<R, 8>; break;
+    RIX_CLEAN(1) RIX_CLEAN(2) RIX_CLEAN(3) RIX_CLEAN(4) RIX_CLEAN(5) RIX_CLEAN(6) RIX_CLEAN(7) RIX_CLEAN(8)
     default: return set_error(RIX_EINVAL, "%d scales", ns);
   }
-  RIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, 0));
+#undef RIX_CLEAN
   // at most four CTAs per SM: enough loads in flight for the sweeps, and
   // every CTA reads every CTA's candidate at each iteration
-  const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ctx->num_sms * std::min(std::max(per_sm, 1), 4),
-                                                                 ceil_div(npix, 256)));
+  const int ntiles = (n / ts) * (n / ts);
+  int nblk = 0;
+  size_t smem = 0;
+  for (int per = 4; per >= 1 && nblk == 0; --per) {
+    const int want = std::min(ctx->num_sms * per, ntiles);
+    smem = (size_t)ceil_div(ntiles, want) * (sizeof(CleanTile<R>) + sizeof(int)) + 16;
+    int per_sm = 0;
+    RIX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem));
+    if (per_sm >= per || (int64_t)per_sm * ctx->num_sms >= want) nblk = want;
+  }
+  if (nblk == 0) return set_error(RIX_EINVAL, "ms-CLEAN kernel does not fit on an SM");
   const size_t comp_bytes = (size_t)cap * (2 * sizeof(int) + sizeof(double)) + 16;
   RIX_TRY(ensure<R>(job, pt.ms_comp, comp_bytes));
-  RIX_TRY(ensure<R>(job, pt.ms_state, 2 * (size_t)nblk * sizeof(Cand<R>) + 64));
+  const size_t reach_bytes = (size_t)ns * (2 * n / ts) * (2 * n / ts) * sizeof(float2);
+  RIX_TRY(ensure<R>(job, pt.ms_state, reach_bytes + 2 * (size_t)nblk * sizeof(Slot<R>) + 64));
   pt.ms_ncomp_cap = cap;
   RIX_CUDA(cudaMemsetAsync(pt.delta.p, 0, npix * sizeof(R), st));
   RIX_CUDA(cudaMemsetAsync(pt.ms_comp.p, 0, comp_bytes, st));
@@ -838,7 +1062,9 @@ int op_msclean(Job* job, int p, const rix_msclean_params* prm, R* delta_out, cud
   ca.P = pt.ms_P.p;
   ca.model = pt.delta.p;
   ca.stencil = stn_dev;
-  ca.slots = pt.ms_state.p;
+  float2* rch = pt.ms_state.as<float2>();
+  ca.reach = rch;
+  ca.slots = pt.ms_state.as<char>() + (reach_bytes + 15) / 16 * 16;
   ca.comp_amp = reinterpret_cast<double*>(cb);
   ca.comp_s = reinterpret_cast<int*>(cb + (size_t)cap * sizeof(double));
   ca.comp_pix = ca.comp_s + cap;
@@ -847,10 +1073,18 @@ int op_msclean(Job* job, int p, const rix_msclean_params* prm, R* delta_out, cud
   RIX_CUDA(cudaMemsetAsync(pt.sync.p, 0, sizeof(unsigned int), st));
   ca.barrier = pt.sync.as<unsigned int>();
   ca.status = job->status.as<int>();
+  {
+    const int64_t warps = (int64_t)ns * (2 * n / ts) * (2 * n / ts);
+    const int blocks = (int)std::min<int64_t>(ceil_div(warps, 8), (int64_t)ctx->num_sms * 8);
+    ::rix::note_launch();
+    if (ts == 32) k_clean_reach<R, 32><<<blocks, 256, 0, st>>>(ca, rch);
+    else k_clean_reach<R, 16><<<blocks, 256, 0, st>>>(ca, rch);
+    RIX_LAUNCH_CHECK();
+  }
   void* args[] = {&ca};
   ::rix::note_launch();
   timing_mark(kTimeMinorLoop, st, true);
-  RIX_CUDA(cudaLaunchCooperativeKernel((const void*)kern, dim3(nblk), dim3(256), args, 0, st));
+  RIX_CUDA(cudaLaunchCooperativeKernel((const void*)kern, dim3(nblk), dim3(256), args, smem, st));
   timing_mark(kTimeMinorLoop, st, false);
   RIX_TRY(publish<R>(job, p, cycle, st));
   if (delta_out) RIX_CUDA(cudaMemcpyAsync(delta_out, pt.delta.p, npix * sizeof(R), cudaMemcpyDeviceToDevice, st));
