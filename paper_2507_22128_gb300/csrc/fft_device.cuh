@@ -144,6 +144,23 @@ __device__ __forceinline__ cplx<R> wscreen(double wp, double nm1) {
   return cmake<cplx<R>>(c, DIR * s);
 }
 
+// exp(DIR 2 pi i w (n-1)) in FP32 with w = wh + wl and n - 1 = m.x + m.y held as
+// pairs of floats (48 bits): the product's leading part is reduced exactly and
+// the rest added, so the turn is as accurate as FP64's after its rounding to
+// float (the leading product is below 2^23 turns, its remainders below 1e-6),
+// at eight FP32 operations instead of five FP64 ones at 1/64 of their rate
+template <int DIR>
+__device__ __forceinline__ float2 wscreen_ff(float wh, float wl, float2 m) {
+  const float p = __fmul_rn(wh, m.x);
+  float e = __fmaf_rn(wh, m.x, -p);
+  e = __fmaf_rn(wh, m.y, e);
+  e = __fmaf_rn(wl, m.x, e);
+  const float fr = (p - rintf(p)) + e;
+  float s, c;
+  sincospif(2.0f * fr, &s, &c);
+  return make_float2(c, DIR * s);
+}
+
 // ------------------------------------------------------ host-side setup ----
 template <typename R>
 const cplx<R>* twiddles(const Ctx* ctx) {

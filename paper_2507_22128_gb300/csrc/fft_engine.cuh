@@ -52,6 +52,7 @@ struct XArgs {
   int M, L, lo, S, nplanes, mode, herm;
   const void* corr;
   const double* nm1;
+  const float2* nm1f;   // n - 1 as pairs of floats (FP32 inverse rows), or null
   double w0, dw;
   const void* screen;   // tabulated corr x phase screen per plane, or null
   int pg;               // inverse rows: planes per grid row y
@@ -771,6 +772,7 @@ __global__ void __launch_bounds__((CropRows<LOGL>::T), (CropRows<LOGL>::kCtas))
     }
     xf_passes<X, R, +1, LOGL, 0>(v, buf, par, tw, tid);
     const double wp = a.w0 + p * a.dw;
+    const float wh = (float)wp, wl = (float)(wp - (double)wh);
     const C* scr = a.mode == kFacPhase && a.screen ? static_cast<const C*>(a.screen) + (int64_t)p * M * M : nullptr;
 #pragma unroll
     for (int it = 0; it < 16 / RADL; ++it) {
@@ -788,7 +790,7 @@ __global__ void __launch_bounds__((CropRows<LOGL>::T), (CropRows<LOGL>::kCtas))
           const C t = scr[pix];
           o += z.x * t.x + z.y * t.y;
         } else if (a.mode == kFacPhase) {
-          const C e = wscreen<R, +1>(wp, a.nm1[pix]);
+          const C e = wscreen_ff<+1>(wh, wl, a.nm1f[pix]);
           o += z.x * e.x - z.y * e.y;
         } else {
           o += z.x;
@@ -880,7 +882,7 @@ constexpr int kMinLogF = 5;
 inline XArgs x_args(const XformGeom& g) {
   XArgs a{};
   a.M = g.M; a.L = g.L; a.lo = g.lo; a.S = g.S; a.nplanes = g.nplanes; a.mode = g.mode; a.herm = g.herm;
-  a.corr = g.corr; a.nm1 = g.nm1; a.w0 = g.w0; a.dw = g.dw; a.screen = g.screen;
+  a.corr = g.corr; a.nm1 = g.nm1; a.nm1f = g.nm1f; a.w0 = g.w0; a.dw = g.dw; a.screen = g.screen;
   a.pg = g.pg > 0 ? g.pg : g.nplanes;
   return a;
 }

@@ -121,9 +121,19 @@ struct CorrArgs {
   const double* ip1;    // 1 / Phi((a - M/2) / Ng), [M]
   int wstack;
   double dw, lo, hi;    // Chebyshev interval of dw (n - 1)
+  int pairs;            // n - 1 stored as a pair of floats (high, low) in the double's place
   int ncheb;            // leading coefficients that count
   double cheb[kCheb];
 };
+
+__device__ __forceinline__ void store_nm1(const CorrArgs& a, double* nm1, int64_t pix, double d) {
+  if (a.pairs) {
+    const float hi = (float)d;
+    reinterpret_cast<float2*>(nm1)[pix] = make_float2(hi, (float)(d - (double)hi));
+  } else {
+    nm1[pix] = d;
+  }
+}
 
 // dw (n - 1) -> n Phi(dw (n - 1)) and n - 1 at squared radius r2 (a Clenshaw
 // sum of the Chebyshev fit of Phi)
@@ -161,7 +171,7 @@ __global__ void k_corrections(CorrArgs a, R* __restrict__ corr, double* __restri
       const double l = (double)(c - h + a.ox) * a.cell, m = (double)(b - h + a.oy) * a.cell;
       double d;
       v /= wfactor(a, __dadd_rn(__dmul_rn(l, l), __dmul_rn(m, m)), &d);
-      nm1[i] = d;
+      store_nm1(a, nm1, i, d);
     }
     corr[i] = (R)v;
   }
@@ -191,17 +201,19 @@ __global__ void k_corrections_sym(CorrArgs a, R* __restrict__ corr, double* __re
         if (cc >= a.M || (w == 1 && cc == c)) continue;
         const int64_t pix = (int64_t)bb * a.M + cc;
         corr[pix] = (R)v;
-        if (a.wstack) nm1[pix] = d;
+        if (a.wstack) store_nm1(a, nm1, pix, d);
       }
     }
   }
 }
 
-// Fills the M x M tables corr and nm1 (w-stacked jobs) for grid side ng,
+// Fills the M x M tables corr and nm1 (w-stacked jobs; `pairs`: n - 1 as pairs
+// of floats, for wscreen_ff) for grid side ng,
 // centred ox, oy cells from the phase centre; the w-correction's Chebyshev
 // fit covers a field of half side `half_px` cells about the phase centre.
 template <typename R>
-int fill_correction(Job* job, int M, int ng, int ox, int oy, int half_px, R* corr, double* nm1, cudaStream_t st) {
+int fill_correction(Job* job, int M, int ng, int ox, int oy, int half_px, R* corr, double* nm1, bool pairs,
+                    cudaStream_t st) {
   static const EsFourier phi;
   const bool ws = job->nw > 0;
   const double cell = job->desc.cell_rad, dw = job->stats.dw;
@@ -211,6 +223,7 @@ int fill_correction(Job* job, int M, int ng, int ox, int oy, int half_px, R* cor
   ca.oy = oy;
   ca.cell = cell;
   ca.wstack = ws;
+  ca.pairs = pairs;
   ca.dw = dw;
   if (ws) {
     // the most negative dw (n - 1) is at the field's corner
@@ -246,10 +259,11 @@ int fill_correction(Job* job, int M, int ng, int ox, int oy, int half_px, R* cor
 }
 
 template <typename R>
-int build_correction(Job* job, int M, int ng, DevBuf& corr, DevBuf& nm1, cudaStream_t st) {
+int build_correction(Job* job, int M, int ng, DevBuf& corr, DevBuf& nm1, bool pairs, cudaStream_t st) {
   RIX_TRY(corr.alloc(job->ctx, (size_t)M * M * sizeof(R)));
   if (job->nw > 0) RIX_TRY(nm1.alloc(job->ctx, (size_t)M * M * sizeof(double)));
-  return fill_correction<R>(job, M, ng, 0, 0, M / 2, corr.as<R>(), job->nw > 0 ? nm1.as<double>() : nullptr, st);
+  return fill_correction<R>(job, M, ng, 0, 0, M / 2, corr.as<R>(), job->nw > 0 ? nm1.as<double>() : nullptr,
+                            pairs, st);
 }
 
 // --------------------------------------------------------------- kernels ----
@@ -838,6 +852,7 @@ XformGeom plane_geom(const Job* job, const Part& pt, bool psf) {
   g.mode = job->nw > 0 ? kFacPhase : kFacReal;
   g.corr = psf ? job->corr_psf.p : job->corr_img.p;
   g.nm1 = psf ? job->nm1_psf.as<double>() : job->nm1_img.as<double>();
+  if (psf && !job->fp64) g.nm1f = job->nm1_psf.as<float2>();
   g.w0 = job->stats.w_min - 0.5 * job->ww * job->stats.dw;
   g.dw = job->stats.dw;
   // the image grid's factors are tabulated once per job (the PSF's grid is
@@ -889,8 +904,8 @@ template <typename R>
 int grid_build_corrections(Job* job, cudaStream_t st) {
   const int n = job->desc.n;
   job->stats.max_dw_nm1 = 0.0;
-  RIX_TRY(build_correction<R>(job, n, job->ng, job->corr_img, job->nm1_img, st));
-  RIX_TRY(build_correction<R>(job, 2 * n, 2 * job->ng, job->corr_psf, job->nm1_psf, st));
+  RIX_TRY(build_correction<R>(job, n, job->ng, job->corr_img, job->nm1_img, false, st));
+  RIX_TRY(build_correction<R>(job, 2 * n, 2 * job->ng, job->corr_psf, job->nm1_psf, sizeof(R) == 4, st));
   if (job->nw > 0) {
     // corr x phase screen of every w-plane on the image grid: read by the
     // row passes of every major cycle instead of forming them in FP64
@@ -1037,9 +1052,10 @@ int op_psf_tiled(Job* job, int p, cudaStream_t st) {
     XformGeom g = g0;
     g.screen = nullptr;
     if (ws) {
-      if ((rc = fill_correction<R>(job, n, job->ng, ox, oy, n, corr, nm1, st)) != RIX_OK) break;
+      if ((rc = fill_correction<R>(job, n, job->ng, ox, oy, n, corr, nm1, sizeof(R) == 4, st)) != RIX_OK) break;
       g.corr = corr;
       g.nm1 = nm1;
+      if (sizeof(R) == 4) g.nm1f = reinterpret_cast<const float2*>(nm1);
     }
     if (cudaMemsetAsync(pt.resid_planes.p, 0, (size_t)np * pt.win_n * pt.win_n * sizeof(cplx<R>), st) != cudaSuccess) {
       rc = set_error(RIX_ECUDA, "memset");

@@ -227,7 +227,9 @@ __device__ __forceinline__ Coords sample_coords(const SampleGeomParams& g, int64
   c.y = __dadd_rn(__dmul_rn(c.vl, g.scale), g.half);
   const double xs = __dadd_rn(c.x, -0.5 * kW);
   const double ys = __dadd_rn(c.y, -0.5 * kW);
-  const bool finite = fabs(xs) < 1e9 && fabs(ys) < 1e9;
+  // |xs|, |ys| < 1e9, by the exponent fields (integer operations)
+  constexpr int kHi1e9 = 0x41cdcd65;
+  const bool finite = (__double2hiint(xs) & 0x7fffffff) < kHi1e9 && (__double2hiint(ys) & 0x7fffffff) < kHi1e9;
   c.ju = finite ? __double2int_ru(xs) : -1;
   c.jv = finite ? __double2int_ru(ys) : -1;
   c.inside = c.ju >= 0 && c.ju + kW <= g.ng && c.jv >= 0 && c.jv + kW <= g.ng;
@@ -242,9 +244,7 @@ __device__ __forceinline__ int sample_plane(const SampleGeomParams& g, int64_t s
   const uint32_t row = (uint32_t)s / (uint32_t)g.nchan;
   const double wl = __dmul_rn(g.uvw[(int64_t)row * 3 + 2], g.inv_lambda[(uint32_t)s - row * (uint32_t)g.nchan]);
   const double tw = div_by(__dadd_rn(wl, -g.w_min), g.dw, g.inv_dw);
-  double p0 = ceil(tw);
-  p0 = fmin(fmax(p0, 0.0), (double)(g.nw - g.ww));
-  return (int)p0;
+  return min(max(__double2int_ru(tw), 0), g.nw - g.ww);
 }
 
 __device__ __forceinline__ unsigned long long ordered_bits(double v) {
@@ -446,58 +446,69 @@ __global__ void k_classify(SampleGeomParams g, int64_t ns, Thresholds th, KeyLay
   }
   if (threadIdx.x == 0) s_out = 0ull;
   __syncthreads();
-  const int lane = threadIdx.x & 31;
-  for (int64_t s0 = (int64_t)blockIdx.x * blockDim.x; s0 < ns; s0 += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t s = s0 + threadIdx.x;
-    const bool live = s < ns;
-    Coords c;
+  // each thread's own partial results over its samples (a reduction per warp
+  // and sample instead was more FP64 and shared-memory work than the samples)
+  int win[kMaxPart][4];
+  unsigned cnt[kMaxPart], outside = 0;
+  double wsum[kMaxPart];
+#pragma unroll
+  for (int p = 0; p < kMaxPart; ++p) {
+    win[p][0] = win[p][2] = INT_MAX;
+    win[p][1] = win[p][3] = INT_MIN;
+    cnt[p] = 0u;
+    wsum[p] = 0.0;
+  }
+  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < ns; s += (int64_t)gridDim.x * blockDim.x) {
+    const Coords c = sample_coords(g, s);
     uint32_t mask = 0, tile = 0;
-    int pju = 0, pjv = 0;
-    float wt = 0.f;
-    if (live) {
-      c = sample_coords(g, s);
-      if (c.inside) {
-        for (int p = 0; p < th.nparts; ++p) {
-          bool ok = true;
-          if (p > 0) ok = ok && (c.q >= th.lo[p]);
-          if (p < th.nparts - 1) ok = ok && (c.q <= th.hi[p]);
-          mask |= (ok ? 1u : 0u) << p;
-        }
-        // first taps on the 4N PSF grid (image 2N): x' = u_l * (dl * 4N) + 2N = 2 x exactly
-        pju = __double2int_ru(__dadd_rn(__dadd_rn(c.x, c.x), -0.5 * kW));
-        pjv = __double2int_ru(__dadd_rn(__dadd_rn(c.y, c.y), -0.5 * kW));
-        tile = ((uint32_t)sample_plane(g, s) << (2 * kl.bt)) | ((uint32_t)(c.jv >> kl.logT) << kl.bt) |
-               (uint32_t)(c.ju >> kl.logT);
+    if (c.inside) {
+      const double wt = o.weight ? (double)o.weight[s] : 1.0;
+      // first taps on the 4N PSF grid (image 2N): x' = u_l * (dl * 4N) + 2N = 2 x exactly
+      const int pju = __double2int_ru(__dadd_rn(__dadd_rn(c.x, c.x), -0.5 * kW));
+      const int pjv = __double2int_ru(__dadd_rn(__dadd_rn(c.y, c.y), -0.5 * kW));
+#pragma unroll
+      for (int p = 0; p < kMaxPart; ++p) {
+        if (p >= th.nparts) break;
+        bool ok = true;
+        if (p > 0) ok = ok && (c.q >= th.lo[p]);
+        if (p < th.nparts - 1) ok = ok && (c.q <= th.hi[p]);
+        if (!ok) continue;
+        mask |= 1u << p;
+        win[p][0] = min(win[p][0], min(c.ju, c.jv));
+        win[p][1] = max(win[p][1], max(c.ju, c.jv));
+        win[p][2] = min(win[p][2], min(pju, pjv));
+        win[p][3] = max(win[p][3], max(pju, pjv));
+        cnt[p] += 1u;
+        wsum[p] += wt;
       }
-      wt = o.weight ? o.weight[s] : 1.0f;
-      if (o.mask_out) o.mask_out[s] = (uint8_t)mask;
-      o.counts[s] = __popc(mask);
-      o.packed[s] = (mask << 24) | tile;
+      tile = ((uint32_t)sample_plane(g, s) << (2 * kl.bt)) | ((uint32_t)(c.jv >> kl.logT) << kl.bt) |
+             (uint32_t)(c.ju >> kl.logT);
+    } else {
+      outside += 1u;
     }
-    const unsigned outside = __ballot_sync(0xffffffffu, live && !c.inside);
-    if (lane == 0 && outside) atomicAdd(&s_out, (unsigned long long)__popc(outside));
-    for (int p = 0; p < th.nparts; ++p) {
-      const bool in = (mask >> p) & 1u;
-      const unsigned bal = __ballot_sync(0xffffffffu, in);
-      if (!bal) continue;
-      int mn = in ? min(c.ju, c.jv) : INT_MAX;
-      int mx = in ? max(c.ju, c.jv) : INT_MIN;
-      int pmn = in ? min(pju, pjv) : INT_MAX;
-      int pmx = in ? max(pju, pjv) : INT_MIN;
-      double w = in ? (double)wt : 0.0;
-      mn = __reduce_min_sync(0xffffffffu, mn);
-      mx = __reduce_max_sync(0xffffffffu, mx);
-      pmn = __reduce_min_sync(0xffffffffu, pmn);
-      pmx = __reduce_max_sync(0xffffffffu, pmx);
-      for (int off = 16; off; off >>= 1) w += __shfl_xor_sync(0xffffffffu, w, off);
-      if (lane == 0) {
-        atomicMin(&s_win[p * 4 + 0], mn);
-        atomicMax(&s_win[p * 4 + 1], mx);
-        atomicMin(&s_win[p * 4 + 2], pmn);
-        atomicMax(&s_win[p * 4 + 3], pmx);
-        atomicAdd(&s_cnt[p], (unsigned long long)__popc(bal));
-        atomicAdd(&s_w[p], w);
-      }
+    if (o.mask_out) o.mask_out[s] = (uint8_t)mask;
+    o.counts[s] = __popc(mask);
+    o.packed[s] = (mask << 24) | tile;
+  }
+  const int lane = threadIdx.x & 31;
+  outside = __reduce_add_sync(0xffffffffu, outside);
+  if (lane == 0 && outside) atomicAdd(&s_out, (unsigned long long)outside);
+#pragma unroll
+  for (int p = 0; p < kMaxPart; ++p) {
+    if (p >= th.nparts) break;
+    const unsigned n = __reduce_add_sync(0xffffffffu, cnt[p]);
+    if (!n) continue;
+    const int mn = __reduce_min_sync(0xffffffffu, win[p][0]), mx = __reduce_max_sync(0xffffffffu, win[p][1]);
+    const int pmn = __reduce_min_sync(0xffffffffu, win[p][2]), pmx = __reduce_max_sync(0xffffffffu, win[p][3]);
+    double w = wsum[p];
+    for (int off = 16; off; off >>= 1) w += __shfl_xor_sync(0xffffffffu, w, off);
+    if (lane == 0) {
+      atomicMin(&s_win[p * 4 + 0], mn);
+      atomicMax(&s_win[p * 4 + 1], mx);
+      atomicMin(&s_win[p * 4 + 2], pmn);
+      atomicMax(&s_win[p * 4 + 3], pmx);
+      atomicAdd(&s_cnt[p], (unsigned long long)n);
+      atomicAdd(&s_w[p], w);
     }
   }
   __syncthreads();
