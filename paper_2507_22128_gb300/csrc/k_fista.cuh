@@ -79,7 +79,12 @@ struct FistaShape {
   static constexpr size_t kFftSmem = 2 * (size_t)B * STRIDE * sizeof(cplx<R>);
   // a unit's slice of Mx (B window columns of length L) or of d (2B rows of
   // N), copied asynchronously while the unit's transform runs
-  static constexpr size_t kStage = (size_t)B * L * sizeof(R);
+  // With the concatenated dictionary they are read where they lie: its wavelet
+  // phases, most of an iteration, gain more from the L1 that the slice's 16 KB
+  // leave (100 iterations of two loops at 512^2 17.8 -> 16.4 ms; Db4 at 1024^2
+  // 20.6 ms staged, 21.4 not)
+  static constexpr bool kStaged = DICT == RIX_DICT_DB4 || sizeof(R) == 8;
+  static constexpr size_t kStage = kStaged ? (size_t)B * L * sizeof(R) : 0;
   static constexpr int KMAX = DICT == RIX_DICT_DB4 ? 8 : kMaxTaps;
   // analysis block side of the fine levels (kTB at the coarse ones; and with
   // FP64, for shared memory)
@@ -302,28 +307,32 @@ __device__ __forceinline__ void rows_fwd_syn_unit(const R* __restrict__ ll, cons
 // forward transform's first pass reads the columns from Tin, the inverse's
 // first pass multiplies by Mx as it loads and its last pass writes the
 // cropped rows to Tout (tb_index layout); the unit's Mx (rows j0 .. j0 + B of the table,
-// contiguous) is copied to shared memory during the forward transform.
-template <typename R, int LOGL>
+// contiguous) is copied to shared memory during the forward transform (kStaged).
+template <typename R, int LOGL, int DICT>
 __device__ __forceinline__ void cols_conv_unit(const cplx<R>* __restrict__ Tin, const R* __restrict__ mx,
                                                cplx<R>* __restrict__ Tout, const cplx<R>* __restrict__ tw,
                                                cplx<R>* s, cplx<R>* s2, R* stage, int u) {
   using C = cplx<R>;
-  using F = FistaShape<R, LOGL>;
+  using F = FistaShape<R, LOGL, DICT>;
   constexpr int L = F::L, N = F::N, H = F::H, B = F::B, S = F::S, STRIDE = F::STRIDE;
   const int j0 = u * B;
   // rows j0 .. j0 + B - 1 < L of the L x L table: in bounds even past S
-  stage_async(stage, mx + (int64_t)j0 * L, (int)F::kStage);
+  if constexpr (F::kStaged) stage_async(stage, mx + (int64_t)j0 * L, (int)F::kStage);
   // centred: position p holds image row (p + N/2) mod L; the pruned half is zero
   auto ld_in = [&](int q, int p) -> C {
     const int j = j0 + q;
     return j < S ? Tin[(int64_t)j * N + ((p + H) & (L - 1))] : cpx<C>(R(0), R(0));
   };
-  auto wait = [] { cp_async_wait_all(); };
+  auto wait = [] {
+    if constexpr (F::kStaged) cp_async_wait_all();
+  };
   C* res = fft_ct<R, -1, LOGL, B, true, false>(s, s2, tw, ld_in, SmemIO{}, wait);
   const C* rin = res;
   auto ld_mul = [&](int q, int p) -> C {
     const C z = rin[q * STRIDE + padi(p)];
-    const R m = stage[q * L + p];
+    R m;
+    if constexpr (F::kStaged) m = stage[q * L + p];
+    else m = mx[(int64_t)(j0 + q) * L + p];
     return cpx<C>(z.x * m, z.y * m);
   };
   auto st_out = [&](int q, int p, const C& v) {
@@ -359,16 +368,16 @@ __device__ __forceinline__ void cols_inv_unit(const cplx<R>* __restrict__ Cs, cp
 // the spectrum given by its window columns k_u in [-N, 0] (T, tb_index
 // layout: the unit's block is contiguous) and Hermitian symmetry; the last
 // pass writes g.
-template <typename R, int LOGL, bool kSubD>
+template <typename R, int LOGL, int DICT, bool kSubD>
 __device__ __forceinline__ void rows_inv_unit(const cplx<R>* __restrict__ T, R* __restrict__ g, R scale,
                                               const R* __restrict__ d, const cplx<R>* __restrict__ tw, cplx<R>* s,
                                               cplx<R>* s2, R* stage, int u) {
   using C = cplx<R>;
-  using F = FistaShape<R, LOGL>;
+  using F = FistaShape<R, LOGL, DICT>;
   constexpr int L = F::L, N = F::N, H = F::H, B = F::B, S = F::S, STRIDE = F::STRIDE;
   const int b0 = u * 2 * B;
-  static_assert(2 * B * N * sizeof(R) <= F::kStage, "d rows exceed the stage");
-  if constexpr (kSubD) stage_async(stage, d + (int64_t)b0 * N, 2 * B * N * (int)sizeof(R));
+  static_assert(!F::kStaged || 2 * B * N * sizeof(R) <= F::kStage, "d rows exceed the stage");
+  if constexpr (kSubD && F::kStaged) stage_async(stage, d + (int64_t)b0 * N, 2 * B * N * (int)sizeof(R));
   // Z = Y_a + i Y_b over all columns: Z[c] from window column c and
   // Z[L - c] = conj Y_a[c] + i conj Y_b[c]; the self-conjugate columns 0 and
   // N keep their real parts (the imaginary parts only feed Im F^-1 Y)
@@ -404,14 +413,19 @@ __device__ __forceinline__ void rows_inv_unit(const cplx<R>* __restrict__ T, R* 
     const R va = z.x * scale, vb = z.y * scale;
     R ga = odd ? -va : va, gb = odd ? vb : -vb;
     if constexpr (kSubD) {
-      ga -= stage[2 * q * N + a];
-      gb -= stage[(2 * q + 1) * N + a];
+      if constexpr (F::kStaged) {
+        ga -= stage[2 * q * N + a];
+        gb -= stage[(2 * q + 1) * N + a];
+      } else {
+        ga -= d[row * N + a];
+        gb -= d[(row + 1) * N + a];
+      }
     }
     g[row * N + a] = ga;
     g[(row + 1) * N + a] = gb;
   };
   auto wait = [] {
-    if constexpr (kSubD) cp_async_wait_all();
+    if constexpr (kSubD && F::kStaged) cp_async_wait_all();
   };
   fft_ct<R, +1, LOGL, B, false, true>(s, s2, tw, SmemIO{}, st_g, wait);
 }
@@ -569,7 +583,7 @@ __device__ __forceinline__ void fista_iterations(const FistaArgs<R>& a, const Fi
   if (!sync()) return;
   for (int u = rank; u < nb * F::kRowUnits; u += stride) {
     const FistaLoop<R>& f = fl[u / F::kRowUnits];
-    rows_inv_unit<R, LOGL, false>(f.tb, f.d, a.gscale, nullptr, f.tw, s, s2, stage, u % F::kRowUnits);
+    rows_inv_unit<R, LOGL, DICT, false>(f.tb, f.d, a.gscale, nullptr, f.tw, s, s2, stage, u % F::kRowUnits);
   }
   if (!sync()) return;
   // FISTA's momentum: t_{k+1} = (1 + sqrt(1 + 4 t_k^2)) / 2, momentum
@@ -614,12 +628,12 @@ __device__ __forceinline__ void fista_iterations(const FistaArgs<R>& a, const Fi
     if (!sync()) return;
     for (int u = rank; u < nb * F::kColUnits; u += stride) {
       const FistaLoop<R>& f = fl[u / F::kColUnits];
-      cols_conv_unit<R, LOGL>(f.ta, f.mx, f.tb, f.tw, s, s2, stage, u % F::kColUnits);
+      cols_conv_unit<R, LOGL, DICT>(f.ta, f.mx, f.tb, f.tw, s, s2, stage, u % F::kColUnits);
     }
     if (!sync()) return;
     for (int u = rank; u < nb * F::kRowUnits; u += stride) {
       const FistaLoop<R>& f = fl[u / F::kRowUnits];
-      rows_inv_unit<R, LOGL, true>(f.tb, f.g, a.gscale, f.d, f.tw, s, s2, stage, u % F::kRowUnits);
+      rows_inv_unit<R, LOGL, DICT, true>(f.tb, f.g, a.gscale, f.d, f.tw, s, s2, stage, u % F::kRowUnits);
     }
     if (!sync()) return;
     const R mom = s_mom;
@@ -805,15 +819,15 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 && LOGL <= 12 ? 2 
     if (stg == 0) {
       cols_inv_unit<R, LOGL>(f.c, f.tb, f.tw, s, s2, u);
     } else if (stg == 1) {
-      rows_inv_unit<R, LOGL, false>(f.tb, f.d, a.gscale, nullptr, f.tw, s, s2, stage, u);
+      rows_inv_unit<R, LOGL, RIX_DICT_DB4, false>(f.tb, f.d, a.gscale, nullptr, f.tw, s, s2, stage, u);
     } else if (kind == kFlowChain) {
       syn_chain_tile<R, T1>(f.y, levels, N, f.tmp, u % kChainNt, u / kChainNt, smem_raw, Db4Taps<R>{});
     } else if (kind == kFlowRowsFwd) {
       rows_fwd_syn_unit<R, LOGL>(levels > 1 ? f.tmp : f.y, f.y, f.ta, f.tw, s, s2, stage, u);
     } else if (kind == kFlowCols) {
-      cols_conv_unit<R, LOGL>(f.ta, f.mx, f.tb, f.tw, s, s2, stage, u);
+      cols_conv_unit<R, LOGL, RIX_DICT_DB4>(f.ta, f.mx, f.tb, f.tw, s, s2, stage, u);
     } else if (kind == kFlowRowsInv) {
-      rows_inv_unit<R, LOGL, true>(f.tb, f.g, a.gscale, f.d, f.tw, s, s2, stage, u);
+      rows_inv_unit<R, LOGL, RIX_DICT_DB4, true>(f.tb, f.g, a.gscale, f.d, f.tw, s, s2, stage, u);
     } else {
       const StepArgs<R> sa{f.alpha, f.y, s_inv_l[b], s_thr[b], s_inv_l[b] != R(0), a.mom ? a.mom[it] : a.mom_tab[it]};
       analysis_unit<R, RIX_DICT_DB4, N>(f, lev, u, sa, smem_raw, a.taps);
@@ -902,9 +916,10 @@ int launch_fista_loop(const Ctx* ctx, const FistaLoop<R>* f, int nb, cudaStream_
     int per_sm = 0;
     RIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFftThreads, smem));
     if (per_sm < 1) return set_error(RIX_EINVAL, "FISTA loop does not fit on an SM (%zu B shared)", smem);
-    // one CTA per SM for a single loop (another partition's loop or gridder fits
-    // beside it); a batch of loops takes up to two
-    const int nblk = ctx->num_sms * std::min(per_sm, nb > 1 ? 2 : 1);
+    // two CTAs per SM for a batch of loops or the loop of an unpartitioned job (50
+    // iterations at 1024^2 3.34 -> 2.52 ms); one for a single partition's loop, so
+    // that another partition's fits beside it
+    const int nblk = ctx->num_sms * std::min(per_sm, nb > 1 || f[0].solo ? 2 : 1);
     if constexpr (DICT == RIX_DICT_DB4) {
       if (nb > 1) {
         // several loops (Db4): the dataflow schedule instead of grid barriers

@@ -1155,6 +1155,7 @@ int fista_prepare(Job* job, int p, const rix_fista_params* prm, FistaLoop<R>* f,
   f->levels = prm->levels;
   f->iters = prm->iters;
   f->dict = prm->dictionary;
+  f->solo = job->n_part == 1;
   f->sched_a = prm->sched_a;
   f->sched_bn = sched_bn;
   if (cat) {

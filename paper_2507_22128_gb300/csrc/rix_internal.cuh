@@ -503,6 +503,7 @@ struct FistaLoop {
   double lambda, lambda_rel;
   int n, levels, iters;
   int dict;                // RIX_DICT_DB4 or RIX_DICT_DB1_8
+  int solo;                // the job's only partition
   double sched_a, sched_bn;   // sched_a > 0: lambda = sched_a * sqrt(state[2]) * sched_bn
   // RIX_DICT_DB1_8 only: member m's coefficients at alpha / y + m N^2, its
   // level buffers at xs / bs + m N^2 (N x N each), W alpha written to delta
