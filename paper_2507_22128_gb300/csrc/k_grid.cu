@@ -626,7 +626,8 @@ __global__ void __launch_bounds__(256) k_tiles_ws(TileArgs a) {
   C* out = static_cast<C*>(a.out);
   const C* vin = static_cast<const C*>(a.vis_in);
   const uint32_t tmask = (1u << a.bt) - 1u;
-  const int per_warp = kWsBatch / nwarps;
+  static_assert(kWsBatch % 8 == 0, "eight warps");
+  constexpr int per_warp = kWsBatch / 8;
 
   for (int64_t it = blockIdx.x; it < a.item_count * a.nsub; it += gridDim.x) {
     const int64_t item = a.item_begin + it / a.nsub;
@@ -677,52 +678,64 @@ __global__ void __launch_bounds__(256) k_tiles_ws(TileArgs a) {
           if (MODE == kGrid || MODE == kResid) { const C v = vin[s]; vre = v.x; vim = v.y; }
           if (MODE == kPsf) vre = R(1);
         }
-        for (int j = 0; j < per_warp && j0 + j < nb; ++j) {
-          const int kou = __shfl_sync(0xffffffffu, ou, j);
-          const int kov = __shfl_sync(0xffffffffu, ov, j);
-          const R kdu = __shfl_sync(0xffffffffu, du, j);
-          const R kdv = __shfl_sync(0xffffffffu, dv, j);
-          const R kdw = __shfl_sync(0xffffffffu, dwo, j);
-          // lanes 0-7: u weights, 8-15: v weights, 16-23: w weights
-          const R kd = lane < 8 ? kdu : (lane < 16 ? kdv : kdw);
-          const R myw = lane < 24 ? es_weight<R>(kd, lane & 7) : R(0);
-          WsRecord<R>& rc = rec[j0 + j];
-          if (lane < 24) rc.w[lane < 8 ? 2 * (lane & 3) + (lane >> 2) : lane] = myw;
-          R accr = R(0), acci = R(0);
-          if constexpr (kUseModel) {
-            R wu[kW];
+        // the 24 kernel weights of each of the warp's entries, all lanes busy
+        // (FP64 exponentials and roots are a third of this kernel's arithmetic)
+        constexpr int kPer = kWsBatch / 8;             // entries per warp
+        static_assert(kPer * 24 % 32 == 0, "whole rounds of weights");
 #pragma unroll
-            for (int i = 0; i < kW; ++i) wu[i] = __shfl_sync(0xffffffffu, myw, i);
-            const int vrow = lane & 7, plh = lane >> 3;
-            const R wv = __shfl_sync(0xffffffffu, myw, 8 + vrow);
+        for (int r = 0; r < kPer * 24 / 32; ++r) {
+          const int e = lane + 32 * r, j = e / 24, tap = e - 24 * j;
+          const R d0 = __shfl_sync(0xffffffffu, du, j), d1 = __shfl_sync(0xffffffffu, dv, j);
+          const R d2 = __shfl_sync(0xffffffffu, dwo, j);
+          const R w = es_weight<R>(tap < 8 ? d0 : (tap < 16 ? d1 : d2), tap & 7);
+          rec[j0 + j].w[tap < 8 ? 2 * (tap & 3) + (tap >> 2) : tap] = w;
+        }
+        __syncwarp();
+        // two entries at a time: independent chains for the FP64 pipe
+        for (int j = 0; j < kPer && j0 + j < nb; j += 2) {
+          R accr[2], acci[2];
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-              const int pl = plh + 4 * r;
-              const R wvw = wv * __shfl_sync(0xffffffffu, myw, 16 + pl);
-              const C* gp = sm_model + pl * PL + kou * SPP + kov + vrow;
-              R sr = R(0), si = R(0);
+          for (int q = 0; q < 2; ++q) {
+            accr[q] = acci[q] = R(0);
+            if constexpr (kUseModel) {
+              const int kou = __shfl_sync(0xffffffffu, ou, j + q), kov = __shfl_sync(0xffffffffu, ov, j + q);
+              const WsRecord<R>& rc = rec[j0 + j + q];
+              const int vrow = lane & 7, plh = lane >> 3;
+              const R wv = rc.w[kW + vrow];
 #pragma unroll
-              for (int i = 0; i < kW; ++i) {
-                const C g = gp[i * SPP];
-                sr += wu[i] * g.x;
-                si += wu[i] * g.y;
+              for (int r = 0; r < 2; ++r) {
+                const int pl = plh + 4 * r;
+                const R wvw = wv * rc.w[2 * kW + pl];
+                const C* gp = sm_model + pl * PL + kou * SPP + kov + vrow;
+                R sr = R(0), si = R(0);
+#pragma unroll
+                for (int i = 0; i < kW; ++i) {
+                  const C g = gp[i * SPP];
+                  const R wu = rc.w[2 * (i & 3) + (i >> 2)];
+                  sr += wu * g.x;
+                  si += wu * g.y;
+                }
+                accr[q] += wvw * sr;
+                acci[q] += wvw * si;
               }
-              accr += wvw * sr;
-              acci += wvw * si;
-            }
-#pragma unroll
-            for (int o = 16; o; o >>= 1) {
-              accr += __shfl_xor_sync(0xffffffffu, accr, o);
-              acci += __shfl_xor_sync(0xffffffffu, acci, o);
             }
           }
-          const R kvr = __shfl_sync(0xffffffffu, vre, j);
-          const R kvi = __shfl_sync(0xffffffffu, vim, j);
-          const R kwt = __shfl_sync(0xffffffffu, wt, j);
-          if (lane == 0) {
-            rc.yr = kwt * (kvr - accr);
-            rc.yi = kwt * (kvi - acci);
-            rc.ouv = (uint32_t)kou | ((uint32_t)kov << 8);
+          if constexpr (kUseModel) {
+#pragma unroll
+            for (int o = 16; o; o >>= 1)
+#pragma unroll
+              for (int q = 0; q < 2; ++q) {
+                accr[q] += __shfl_xor_sync(0xffffffffu, accr[q], o);
+                acci[q] += __shfl_xor_sync(0xffffffffu, acci[q], o);
+              }
+          }
+          // lane j + q holds its entry's data; lanes past nb wrote no record
+          const int q = lane - j;
+          if (q >= 0 && q < 2 && j0 + lane < nb) {
+            WsRecord<R>& rc = rec[j0 + lane];
+            rc.yr = wt * (vre - (q ? accr[1] : accr[0]));
+            rc.yi = wt * (vim - (q ? acci[1] : acci[0]));
+            rc.ouv = (uint32_t)ou | ((uint32_t)ov << 8);
           }
         }
       }

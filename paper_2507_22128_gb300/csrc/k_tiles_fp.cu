@@ -474,9 +474,10 @@ __device__ __forceinline__ float2 bfly(bool hi, float2 lo_v, float2 hi_v, int ma
   return make_float2(keep.x + __shfl_xor_sync(kFull, send.x, mask), keep.y + __shfl_xor_sync(kFull, send.y, mask));
 }
 
-// 16-byte asynchronous global -> shared copy (cp.async, cached at L2 only)
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+// 16-byte asynchronous global -> shared copy (cp.async, cached at L2 only) of
+// `bytes` (16, or 0: nothing is read and the destination is zeroed)
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(bytes) : "memory");
 }
 
 // per warp: a batch's records ({du, dv, dw, tap}; {w re v, w im v, w, 0}, the
@@ -624,13 +625,10 @@ __global__ void __launch_bounds__(kFpThreads, 2)
     // the one slot (its last batch's weights are formed), the visibilities
     // into slot `sl`; entries past nb are zero (zero weight and data)
     auto fetch = [&](uint32_t eb, int nb, int sl) {
-      if (lane < nb) {
-        cp_async16(&ws.g[lane], a.geom + eb + lane);
-        if constexpr (kSpread) cp_async16(&ws.y[sl][lane], a.ysamp + eb + lane);
-      } else {
-        ws.g[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if constexpr (kSpread) ws.y[sl][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
+      const int bytes = lane < nb ? 16 : 0;
+      const uint32_t e = eb + (uint32_t)min(lane, nb - 1);
+      cp_async16(&ws.g[lane], a.geom + e, bytes);
+      if constexpr (kSpread) cp_async16(&ws.y[sl][lane], a.ysamp + e, bytes);
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
 
@@ -663,7 +661,7 @@ __global__ void __launch_bounds__(kFpThreads, 2)
         __syncwarp();
         const uint32_t ouv = __float_as_uint(ws.g[0].w);
         {
-          if constexpr (MODE == kResid) {
+          if constexpr (MODE == kResid && !BATCH) {
             // an entry per lane (fewer registers live in the residual mode:
             // 11.14 against 11.45 ms for ten launches of the 1024^2 job, where
             // the gridding mode takes 1.97 against 1.86 ms)
