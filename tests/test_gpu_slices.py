@@ -1,5 +1,5 @@
-"""Work items cut into slices (k_tiles, k_tiles_ws): sample counts on both
-sides of the slice and item sizes, all in one or two uv tiles, degrid and grid
+"""Work items cut into slices (k_tiles, k_tiles_ws) or chunks (k_tiles_fp): sample
+counts on both sides of the slice and item sizes, all in one or two uv tiles, degrid and grid
 of every precision and w-mode that uses them, against the direct DFT.
 
 Tolerances (relative L2): FP32 1e-5 (kernel error 1e-7, a few roundings per
@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 CELL = np.pi / 180 / 3600
 
 
-@pytest.mark.parametrize("prec,planes,tile", [(0, 0, 16), (0, 0, 32), (1, 0, 16), (1, 9, 16)])
+@pytest.mark.parametrize("prec,planes,tile", [(0, 0, 16), (0, 0, 32), (0, 9, 16), (1, 0, 16), (1, 9, 16)])
 @pytest.mark.parametrize("ns", [1, 63, 64, 65, 257, 2047, 2048, 2049, 4999])
 def test_crowded_tile(ns, prec, planes, tile):
     need_gpu()
