@@ -43,12 +43,26 @@
 namespace rix {
 namespace {
 
-// analysis block side: 32 at the fine levels with FP32 and Db4 (at least 256
-// blocks per loop; with fewer, the smaller blocks keep more CTAs busy), kTB
-// otherwise
+// analysis block side: 32 at the fine levels with FP32 (at least 256 blocks per
+// loop with Db4, 128 with the concatenated dictionary; with fewer, the smaller
+// blocks keep more CTAs busy), kTB otherwise.  A unit's time is the latency of
+// its chain (copies, rows, columns, with a barrier between), nearly the same
+// for 2 and for 16 taps, so fewer and larger units are faster: levels 0 and 1 of
+// eight members of two 512^2 loops 50 + 14 us with blocks of 16, 42 + 10 us
 template <typename R, int DICT>
 __host__ __device__ constexpr int ana_fine_block() {
-  return sizeof(R) == 4 && DICT == RIX_DICT_DB4 ? 32 : kTB;
+  return sizeof(R) == 4 ? 32 : kTB;
+}
+// likewise the synthesis levels of the concatenated dictionary: blocks of 64
+// from 128 of them per loop on (level 0 of two 512^2 loops 33 -> 25 us)
+template <typename R, int DICT>
+__host__ __device__ constexpr int syn_fine_block() {
+  return sizeof(R) == 4 && DICT != RIX_DICT_DB4 ? 64 : kTS;
+}
+template <typename R, int DICT>
+__device__ __forceinline__ int syn_block(int n) {
+  constexpr int TSF = syn_fine_block<R, DICT>();
+  return TSF != kTS && 8 * (n / TSF) * (n / TSF) >= 128 ? TSF : kTS;
 }
 // block side of the chained coarse synthesis (the level-1 output per unit)
 template <typename R>
@@ -59,7 +73,8 @@ __host__ __device__ constexpr int chain_block() {
 template <typename R, int DICT>
 __device__ __forceinline__ int ana_block(int h) {
   constexpr int TBF = ana_fine_block<R, DICT>();
-  return (TBF != kTB && (h / TBF) * (h / TBF) >= 256) ? TBF : kTB;
+  constexpr int kMin = DICT == RIX_DICT_DB4 ? 256 : 128 / 8;   // blocks per member
+  return (TBF != kTB && (h / TBF) * (h / TBF) >= kMin) ? TBF : kTB;
 }
 
 template <typename R, int LOGL, int DICT = RIX_DICT_DB4>
@@ -92,8 +107,9 @@ struct FistaShape {
   static constexpr size_t kDwtSmem = sizeof(DwtSmem<R, TBF, KMAX>) > sizeof(DwtSmem<R, kTB, KMAX>)
                                          ? sizeof(DwtSmem<R, TBF, KMAX>)
                                          : sizeof(DwtSmem<R, kTB, KMAX>);
-  static constexpr size_t kIdwtSmem = sizeof(IdwtSmem<R, KMAX>) > chain_smem_bytes<R, chain_block<R>(), 8>()
-                                          ? sizeof(IdwtSmem<R, KMAX>)
+  static constexpr int TSF = syn_fine_block<R, DICT>();
+  static constexpr size_t kIdwtSmem = sizeof(IdwtSmem<R, KMAX, TSF>) > chain_smem_bytes<R, chain_block<R>(), 8>()
+                                          ? sizeof(IdwtSmem<R, KMAX, TSF>)
                                           : chain_smem_bytes<R, chain_block<R>(), 8>();
   static constexpr size_t kWavSmem = kDwtSmem > kIdwtSmem ? kDwtSmem : kIdwtSmem;
   static constexpr size_t kSmem = kFftSmem + kStage > kWavSmem ? kFftSmem + kStage : kWavSmem;
@@ -157,27 +173,38 @@ __device__ __forceinline__ void rows_fwd_unit(const R* __restrict__ x, int64_t x
   const int b0 = u * 2 * B;
   // complex row q = x[b0 + 2q] + i x[b0 + 2q + 1], centred: pixel a sits at
   // grid column (a - N/2) mod L with sign (-1)^(a + b)
-  constexpr int NE = B * N;
+  // read in 16-byte chunks: with NSUM images a value is NSUM loads
+  constexpr int CH = kChunk<R>;
+  constexpr int NE = B * N / CH;
   constexpr int NLD = (NE + kFftThreads - 1) / kFftThreads;
-  R va[NLD], vb[NLD];
+  static_assert(N % CH == 0, "whole chunks to a row");
+  R va[NLD][CH], vb[NLD][CH];
 #pragma unroll
   for (int k = 0; k < NLD; ++k) {
     const int e = threadIdx.x + k * kFftThreads;
     if (NE % kFftThreads == 0 || e < NE) {
-      const int q = e / N, a = e % N;
-      const int64_t row = b0 + 2 * q;
+      const R* p = x + (int64_t)(b0 + 2 * (e / (N / CH))) * N + e % (N / CH) * CH;
       if constexpr (NSUM == 1) {
-        va[k] = x[row * N + a];
-        vb[k] = x[(row + 1) * N + a];
+        ld_chunk(p, va[k]);
+        ld_chunk(p + N, vb[k]);
       } else {
-        R sa = R(0), sb = R(0);
+        R sa[CH] = {}, sb[CH] = {};
 #pragma unroll
         for (int m = 0; m < NSUM; ++m) {
-          sa += x[m * xstride + row * N + a];
-          sb += x[m * xstride + (row + 1) * N + a];
+          R qa[CH], qb[CH];
+          ld_chunk(p + m * xstride, qa);
+          ld_chunk(p + m * xstride + N, qb);
+#pragma unroll
+          for (int j = 0; j < CH; ++j) {
+            sa[j] += qa[j];
+            sb[j] += qb[j];
+          }
         }
-        va[k] = xscale * sa;
-        vb[k] = xscale * sb;
+#pragma unroll
+        for (int j = 0; j < CH; ++j) {
+          va[k][j] = xscale * sa[j];
+          vb[k][j] = xscale * sb[j];
+        }
       }
     }
   }
@@ -185,9 +212,13 @@ __device__ __forceinline__ void rows_fwd_unit(const R* __restrict__ x, int64_t x
   for (int k = 0; k < NLD; ++k) {
     const int e = threadIdx.x + k * kFftThreads;
     if (NE % kFftThreads == 0 || e < NE) {
-      const int q = e / N, a = e % N;
-      const bool odd = (a + b0) & 1;               // b0 + 2q has the parity of b0
-      s[q * STRIDE + padi((a - H) & (L - 1))] = cpx<C>(odd ? -va[k] : va[k], odd ? vb[k] : -vb[k]);
+      const int q = e / (N / CH), a0 = e % (N / CH) * CH;
+#pragma unroll
+      for (int j = 0; j < CH; ++j) {
+        const bool odd = (j + b0) & 1;             // a0 is even and b0 + 2q has the parity of b0
+        s[q * STRIDE + padi((a0 + j - H) & (L - 1))] =
+            cpx<C>(odd ? -va[k][j] : va[k][j], odd ? vb[k][j] : -vb[k][j]);
+      }
     }
   }
   __syncthreads();
@@ -432,17 +463,17 @@ __device__ __forceinline__ void rows_inv_unit(const cplx<R>* __restrict__ T, R* 
 
 // member MM of the concatenated dictionary (db_{MM+1}, 2 (MM + 1) taps),
 // out of line: each member's tile gets its own register allocation
-template <typename R, int MM>
+template <typename R, int MM, int TS>
 __device__ __noinline__ void syn_member(const R* ll, const R* cm, int n, R* dst, int N, int bx, int by,
                                         unsigned char* smem, const R* taps) {
-  auto& ism = *reinterpret_cast<IdwtSmem<R, 2 * (MM + 1)>*>(smem);
-  idwt_tile<R>(ll, cm, n, dst, N, bx, by, ism, RefTaps<R, 2 * (MM + 1)>{taps});
+  auto& ism = *reinterpret_cast<IdwtSmem<R, 2 * (MM + 1), TS>*>(smem);
+  idwt_tile<R, true, TS>(ll, cm, n, dst, N, bx, by, ism, RefTaps<R, 2 * (MM + 1)>{taps});
 }
-template <typename R, int MM>
+template <typename R, int MM, int TB>
 __device__ __noinline__ void ana_member(const R* src, int n, R* dst, int N, int last, const StepArgs<R>& sm,
                                         int bx, int by, unsigned char* smem, const R* taps) {
-  auto& dsm = *reinterpret_cast<DwtSmem<R, kTB, 2 * (MM + 1)>*>(smem);
-  dwt_tile<R, kTB, true>(src, N, n, nullptr, dst, N, last, sm, bx, by, dsm, RefTaps<R, 2 * (MM + 1)>{taps});
+  auto& dsm = *reinterpret_cast<DwtSmem<R, TB, 2 * (MM + 1)>*>(smem);
+  dwt_tile<R, TB, true>(src, N, n, nullptr, dst, N, last, sm, bx, by, dsm, RefTaps<R, 2 * (MM + 1)>{taps});
 }
 
 // iterations whose FISTA momentum travels in the launch arguments
@@ -461,6 +492,7 @@ struct FistaArgs {
   unsigned int* done;
   const R* mom;           // device table, or null: mom_tab holds the iterations
   R mom_tab[kMomTab];
+  double t_tab;           // t after those iterations (or after all, if fewer)
 };
 
 // units of one wavelet level of one loop: tiles of side `tile` over an n x n
@@ -477,13 +509,13 @@ __device__ __forceinline__ int level_units(int n, int tile) {
 template <typename R, int DICT, int N>
 __device__ __forceinline__ void synthesis_unit(const FistaLoop<R>& f, const R* coef, int l, int t,
                                                unsigned char* smem, const R (&taps)[8][16]) {
-  const int n = N >> l, nt = (n + kTS - 1) / kTS, per = nt * nt;
+  const int n = N >> l, ts = syn_block<R, DICT>(n), nt = (n + ts - 1) / ts, per = nt * nt;
   const bool top = l == f.levels - 1;
   if constexpr (DICT == RIX_DICT_DB4) {
     const R* ll = top ? coef : (((l + 1) & 1) ? f.tmp : f.x);
     R* dst = (l & 1) ? f.tmp : f.x;
     auto& ism = *reinterpret_cast<IdwtSmem<R, 8>*>(smem);
-    idwt_tile<R>(ll, coef, n, dst, N, t % nt, t / nt, ism, Db4Taps<R>{});
+    idwt_tile<R, true>(ll, coef, n, dst, N, t % nt, t / nt, ism, Db4Taps<R>{});
   } else {
     const int64_t NN = (int64_t)N * N;
     const int m = t / per, tt = t - m * per;
@@ -493,8 +525,12 @@ __device__ __forceinline__ void synthesis_unit(const FistaLoop<R>& f, const R* c
     const R* ll = top ? cm : (((l + 1) & 1) ? bm : am);
     R* dst = (l & 1) ? bm : am;
     const int bx = tt % nt, by = tt / nt;
+    constexpr int TSF = syn_fine_block<R, DICT>();
 #define RIX_SYN(MM)                                                                                     \
-  case MM: syn_member<R, MM>(ll, cm, n, dst, N, bx, by, smem, taps[MM]); break;
+  case MM:                                                                                              \
+    if (TSF != kTS && ts == TSF) syn_member<R, MM, TSF>(ll, cm, n, dst, N, bx, by, smem, taps[MM]);     \
+    else syn_member<R, MM, kTS>(ll, cm, n, dst, N, bx, by, smem, taps[MM]);                             \
+    break;
     switch (m) { RIX_SYN(0) RIX_SYN(1) RIX_SYN(2) RIX_SYN(3) RIX_SYN(4) RIX_SYN(5) RIX_SYN(6) RIX_SYN(7) }
 #undef RIX_SYN
   }
@@ -530,8 +566,12 @@ __device__ __forceinline__ void analysis_unit(const FistaLoop<R>& f, int l, int 
     sm.alpha += m * NN;
     sm.y += m * NN;
     const int bx = tt % nt, by = tt / nt;
+    constexpr int TBF = ana_fine_block<R, DICT>();
 #define RIX_ANA(MM)                                                                                     \
-  case MM: ana_member<R, MM>(src, n, dst, N, last, sm, bx, by, smem, taps[MM]); break;
+  case MM:                                                                                              \
+    if (TBF != kTB && tb == TBF) ana_member<R, MM, TBF>(src, n, dst, N, last, sm, bx, by, smem, taps[MM]); \
+    else ana_member<R, MM, kTB>(src, n, dst, N, last, sm, bx, by, smem, taps[MM]);                      \
+    break;
     switch (m) { RIX_ANA(0) RIX_ANA(1) RIX_ANA(2) RIX_ANA(3) RIX_ANA(4) RIX_ANA(5) RIX_ANA(6) RIX_ANA(7) }
 #undef RIX_ANA
   }
@@ -586,15 +626,15 @@ __device__ __forceinline__ void fista_iterations(const FistaArgs<R>& a, const Fi
     rows_inv_unit<R, LOGL, DICT, false>(f.tb, f.d, a.gscale, nullptr, f.tw, s, s2, stage, u % F::kRowUnits);
   }
   if (!sync()) return;
-  // FISTA's momentum: t_{k+1} = (1 + sqrt(1 + 4 t_k^2)) / 2, momentum
-  // (t_k - 1) / t_{k+1}, each operation rounded on its own; one thread per
-  // CTA forms it (FP64 square root and division at 1/64 of the FP32 rate),
-  // at the start of the iteration: the grid barriers before the analysis
+  // FISTA's momentum comes with the launch for the first kMomTab iterations
+  // (an FP64 root and division at the head of an iteration held its first phase
+  // up by about a microsecond and a half); beyond them one thread per CTA forms
+  // it at the start of the iteration, and the barriers before the analysis
   // phases publish it to the CTA
   __shared__ R s_mom;
-  double t = 1.0;
+  double t = a.t_tab;
   for (int it = 0; it < f0.iters; ++it) {
-    if (threadIdx.x == 0) {
+    if (it >= kMomTab && threadIdx.x == 0) {
       const double tn = __dmul_rn(0.5, __dadd_rn(1.0, __dsqrt_rn(__dadd_rn(1.0, __dmul_rn(__dmul_rn(4.0, t), t)))));
       s_mom = (R)__ddiv_rn(__dadd_rn(t, -1.0), tn);
       t = tn;
@@ -604,7 +644,7 @@ __device__ __forceinline__ void fista_iterations(const FistaArgs<R>& a, const Fi
     // row transforms
     if constexpr (kCat) {
       for (int l = levels - 1; l >= 0; --l) {
-        const int per = level_units<DICT>(N >> l, kTS);
+        const int per = level_units<DICT>(N >> l, syn_block<R, DICT>(N >> l));
         for (int u = rank; u < nb * per; u += stride) {
           const FistaLoop<R>& f = fl[u / per];
           synthesis_unit<R, DICT, N>(f, f.y, l, u % per, smem_raw, a.taps);
@@ -636,7 +676,7 @@ __device__ __forceinline__ void fista_iterations(const FistaArgs<R>& a, const Fi
       rows_inv_unit<R, LOGL, DICT, true>(f.tb, f.g, a.gscale, f.d, f.tw, s, s2, stage, u % F::kRowUnits);
     }
     if (!sync()) return;
-    const R mom = s_mom;
+    const R mom = it < kMomTab ? a.mom_tab[it] : s_mom;
     for (int l = 0; l < levels; ++l) {
       const int per = level_units<DICT>((N >> l) / 2, ana_block<R, DICT>((N >> l) / 2));
       for (int u = rank; u < nb * per; u += stride) {
@@ -651,7 +691,7 @@ __device__ __forceinline__ void fista_iterations(const FistaArgs<R>& a, const Fi
   if constexpr (kCat) {
     // each loop's image W alpha: the members' syntheses, summed
     for (int l = levels - 1; l >= 0; --l) {
-      const int per = level_units<DICT>(N >> l, kTS);
+      const int per = level_units<DICT>(N >> l, syn_block<R, DICT>(N >> l));
       for (int u = rank; u < nb * per; u += stride) {
         const FistaLoop<R>& f = fl[u / per];
         synthesis_unit<R, DICT, N>(f, f.alpha, l, u % per, smem_raw, a.taps);
@@ -851,9 +891,10 @@ __global__ void k_mom_table(int iters, R* mom) {
 }
 
 // the same sequence on the host, each operation rounded on its own
-// (volatile temporaries keep the compiler from contracting them)
+// (volatile temporaries keep the compiler from contracting them); returns the
+// t after them
 template <typename R>
-void mom_host(int iters, R* mom) {
+double mom_host(int iters, R* mom) {
   double t = 1.0;
   for (int it = 0; it < iters; ++it) {
     volatile double a = 4.0 * t;
@@ -867,6 +908,7 @@ void mom_host(int iters, R* mom) {
     mom[it] = (R)m;
     t = tn;
   }
+  return t;
 }
 
 template <typename R, int LOGL, int DICT>
@@ -889,6 +931,7 @@ int launch_fista_loop(const Ctx* ctx, const FistaLoop<R>* f, int nb, cudaStream_
       for (int i = 0; i < 16; ++i) args.taps[m][i] = i < k ? (R)h[i] : R(0);
     }
   }
+  args.t_tab = mom_host<R>(std::min(f[0].iters, kMomTab), args.mom_tab);
   if constexpr (LOGL <= kClusterLogL) {
     auto ck = k_fista_cluster<R, LOGL, DICT>;
     RIX_CUDA(cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -946,10 +989,7 @@ int launch_fista_loop(const Ctx* ctx, const FistaLoop<R>* f, int nb, cudaStream_
         } else {
           args.ticket = ctl;
           args.done = ctl + 1;
-          if (f[0].iters <= kMomTab) {
-            mom_host<R>(f[0].iters, args.mom_tab);
-            args.mom = nullptr;
-          } else {
+          if (f[0].iters > kMomTab) {
             ::rix::note_launch();
             k_mom_table<R><<<1, 1, 0, st>>>(f[0].iters, mom);
             args.mom = mom;

@@ -266,7 +266,7 @@ template <typename R>
 __global__ void __launch_bounds__(256) k_idwt_level(const R* __restrict__ llin, const R* __restrict__ coef, int n,
                                                     R* __restrict__ out, int ld) {
   __shared__ IdwtSmem<R, 8> sm;
-  idwt_tile<R>(llin, coef, n, out, ld, blockIdx.x, blockIdx.y, sm, Db4Taps<R>{});
+  idwt_tile<R, false>(llin, coef, n, out, ld, blockIdx.x, blockIdx.y, sm, Db4Taps<R>{});
 }
 
 // coefficients c (N x N) -> image out; tmp: N x N scratch.  Levels are

@@ -73,6 +73,17 @@ constexpr int kTB = 16;                      // the smaller block side
 constexpr int kMaxTaps = 16;                 // db8
 template <int TB, int K> constexpr int tin_side() { return 2 * TB + K - 2; }
 
+// 16 bytes: four floats or two doubles
+template <typename R> constexpr int kChunk = 16 / (int)sizeof(R);
+__device__ __forceinline__ void ld_chunk(const float* p, float* w) {
+  const float4 q = *reinterpret_cast<const float4*>(p);
+  w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w;
+}
+__device__ __forceinline__ void ld_chunk(const double* p, double* w) {
+  const double2 q = *reinterpret_cast<const double2*>(p);
+  w[0] = q.x; w[1] = q.y;
+}
+
 // FISTA step fused into the analysis of the gradient (Beck & Teboulle 2009):
 // at each final coefficient c = s g:  a' = S_{lam/L}(y - c/L),
 // y = a' + mom (a' - a),  a = a'   (s: the dictionary's scale; inv_l folds it)
@@ -88,7 +99,10 @@ struct StepArgs {
 template <typename R, int TB, int K>
 struct DwtSmem {
   static constexpr int TIN = tin_side<TB, K>();
-  R tin[TIN][TIN + 1];
+  // input rows in 16-byte chunks, an odd number to the row: a warp that reads
+  // a chunk of 32 rows meets no bank conflict
+  static constexpr int NCH = (TIN + kChunk<R> - 1) / kChunk<R>;
+  alignas(16) R tin[TIN][(NCH | 1) * kChunk<R>];
   R trow[TIN][2 * TB + 1];             // [input row][lo x | hi x]
   alignas(16) R ys[4][TB * TB];        // step inputs per quadrant, [row][column] of the block
   alignas(16) R as[4][TB * TB];
@@ -122,9 +136,15 @@ __device__ __forceinline__ void dwt_tile(const R* __restrict__ src, int lds, int
       }
     }
   }
-  for (int t = threadIdx.x; t < TIN * TIN; t += blockDim.x) {
-    const int r = t / TIN, c = t - r * TIN;
-    cp_async<(int)sizeof(R)>(&tin[r][c], src + (int64_t)((2 * y0 + r) & (n - 1)) * lds + ((2 * x0 + c) & (n - 1)));
+  // the input in 16-byte chunks (src 16-byte aligned, lds and n multiples of
+  // the chunk, so none straddles the period); the last may reach past the tile.
+  // A copy per value was a third of the tile's instructions (with the vector
+  // reads of the row pass, 57 -> 50 us for level 0 of two 512^2 loops and
+  // eight filters)
+  constexpr int NCH = DwtSmem<R, TB, K>::NCH;
+  for (int t = threadIdx.x; t < TIN * NCH; t += blockDim.x) {
+    const int r = t / NCH, c = (t - r * NCH) * kChunk<R>;
+    cp_async16(&tin[r][c], src + (int64_t)((2 * y0 + r) & (n - 1)) * lds + ((2 * x0 + c) & (n - 1)));
   }
   cp_async_wait_all();
   __syncthreads();
@@ -135,9 +155,10 @@ __device__ __forceinline__ void dwt_tile(const R* __restrict__ src, int lds, int
   constexpr int XG = 4;
   for (int t = threadIdx.x; t < TIN * (TB / XG); t += blockDim.x) {
     const int r = t % TIN, xx = (t / TIN) * XG;
-    R w[2 * XG + K - 2];
+    constexpr int NW = (2 * XG + K - 2 + kChunk<R> - 1) / kChunk<R>;
+    R w[NW * kChunk<R>];
 #pragma unroll
-    for (int i = 0; i < 2 * XG + K - 2; ++i) w[i] = tin[r][2 * xx + i];
+    for (int i = 0; i < NW; ++i) ld_chunk(&tin[r][2 * xx + kChunk<R> * i], w + kChunk<R> * i);
 #pragma unroll
     for (int u = 0; u < XG; ++u) {
       R a = R(0), d = R(0);
@@ -199,49 +220,82 @@ __device__ __forceinline__ void dwt_tile(const R* __restrict__ src, int lds, int
 
 // ------------------------------------------------------- synthesis level ----
 // out (n x n, ld) from the LL block `llin` (ld) and the detail subbands of
-// `coef` (ld); a CTA owns a kTS x kTS output block.
+// `coef` (ld); a CTA owns a TS x TS output block.
 constexpr int kTS = 32;
-template <int K> constexpr int rk_side() { return kTS / 2 + K / 2; }
+template <int K, int TS> constexpr int rk_side() { return TS / 2 + K / 2; }
 
-template <typename R, int K>
+template <typename R, int K, int TS = kTS>
 struct IdwtSmem {
-  static constexpr int RK = rk_side<K>();
+  static constexpr int RK = rk_side<K, TS>();
   R cq[4][RK][RK + 1];         // quadrant tiles: LL, row-high, col-high, HH
-  R tr[2][RK][kTS + 1];        // after row synthesis: [column half][coef row][c]
+  R tr[2][RK][TS + 1];        // after row synthesis: [column half][coef row][c]
 };
 
-template <typename R, typename TAPS>
+// kVec: llin and coef are 16-byte aligned and ld and n / 2 multiples of the
+// 16-byte chunk, and the quadrant tiles are read in chunks (from the chunk that
+// holds their first column): a quarter of the load instructions, 42 -> 33 us for
+// the last level of two 512^2 loops and eight filters
+template <typename R, bool kVec, int TS = kTS, typename TAPS>
 __device__ __forceinline__ void idwt_tile(const R* __restrict__ llin, const R* __restrict__ coef, int n,
-                                          R* __restrict__ out, int ld, int bx, int by, IdwtSmem<R, TAPS::K>& sm,
+                                          R* __restrict__ out, int ld, int bx, int by, IdwtSmem<R, TAPS::K, TS>& sm,
                                           const TAPS& tp) {
   constexpr int K = TAPS::K;
-  constexpr int RK = rk_side<K>();
+  constexpr int RK = rk_side<K, TS>();
   auto& cq = sm.cq;
   auto& tr = sm.tr;
   const int h = n / 2;
-  const int m0 = by * kTS, c0 = bx * kTS;
+  const int m0 = by * TS, c0 = bx * TS;
   // output m uses coefficients (m - i) / 2 for the taps i of its parity
   const int kb_m = (m0 >> 1) - K / 2, kb_c = (c0 >> 1) - K / 2;
-  constexpr int NLD = (4 * RK * RK + 255) / 256;
-  R v[NLD];
+  if constexpr (kVec) {
+    constexpr int CH = kChunk<R>;
+    constexpr int M = (K / 2 + CH - 1) / CH * CH, SKIP = M - K / 2;   // columns read left of c0 / 2, before kb_c
+    constexpr int NCH = (M + TS / 2) / CH;
+    constexpr int NLD = (4 * RK * NCH + 255) / 256;
+    R v[NLD][CH];
 #pragma unroll
-  for (int k = 0; k < NLD; ++k) {
-    const int t = threadIdx.x + 256 * k;
-    if (t < 4 * RK * RK) {
-      const int q = t / (RK * RK), rem = t - q * RK * RK;
-      const int rk = rem / RK, ck = rem - rk * RK;
-      const int km = (kb_m + rk) & (h - 1), kc = (kb_c + ck) & (h - 1);   // periodic; h a power of two
-      const int cy = q >> 1, cx = q & 1;
-      v[k] = (q == 0) ? llin[(int64_t)km * ld + kc] : coef[(int64_t)(cy * h + km) * ld + (cx * h + kc)];
+    for (int k = 0; k < NLD; ++k) {
+      const int t = threadIdx.x + 256 * k;
+      if (t < 4 * RK * NCH) {
+        const int row = t / NCH, q = row / RK, rk = row - q * RK;
+        const int km = (kb_m + rk) & (h - 1), kc = ((c0 >> 1) - M + CH * (t - row * NCH)) & (h - 1);
+        ld_chunk(q == 0 ? llin + (int64_t)km * ld + kc
+                        : coef + (int64_t)((q >> 1) * h + km) * ld + ((q & 1) * h + kc), v[k]);
+      }
     }
-  }
 #pragma unroll
-  for (int k = 0; k < NLD; ++k) {
-    const int t = threadIdx.x + 256 * k;
-    if (t < 4 * RK * RK) {
-      const int q = t / (RK * RK), rem = t - q * RK * RK;
-      const int rk = rem / RK, ck = rem - rk * RK;
-      cq[q][rk][ck] = v[k];
+    for (int k = 0; k < NLD; ++k) {
+      const int t = threadIdx.x + 256 * k;
+      if (t < 4 * RK * NCH) {
+        const int row = t / NCH, q = row / RK, rk = row - q * RK;
+        const int ck = CH * (t - row * NCH) - SKIP;
+#pragma unroll
+        for (int j = 0; j < CH; ++j)
+          if (j >= SKIP || ck + j >= 0) cq[q][rk][ck + j] = v[k][j];
+      }
+    }
+  } else {
+    constexpr int NLD = (4 * RK * RK + 255) / 256;
+    R v[NLD];
+#pragma unroll
+    for (int k = 0; k < NLD; ++k) {
+      const int t = threadIdx.x + 256 * k;
+      if (t < 4 * RK * RK) {
+        const int q = t / (RK * RK), rem = t - q * RK * RK;
+        const int rk = rem / RK, ck = rem - rk * RK;
+        const int km = (kb_m + rk) & (h - 1), kc = (kb_c + ck) & (h - 1);   // periodic; h a power of two
+        const int cy = q >> 1, cx = q & 1;
+        v[k] = (q == 0) ? llin[(int64_t)km * ld + kc] : coef[(int64_t)(cy * h + km) * ld + (cx * h + kc)];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < NLD; ++k) {
+      const int t = threadIdx.x + 256 * k;
+      if (t < 4 * RK * RK) {
+        const int q = t / (RK * RK), rem = t - q * RK * RK;
+        const int rk = rem / RK, ck = rem - rk * RK;
+        cq[q][rk][ck] = v[k];
+      }
     }
   }
   __syncthreads();
@@ -250,7 +304,7 @@ __device__ __forceinline__ void idwt_tile(const R* __restrict__ llin, const R* _
   // adjacent c (two of each parity) from the K/2 + 1 coefficients they share
   // in each of the two subbands (c0 and m0 are even).
   constexpr int HK = K / 2;
-  for (int t = threadIdx.x; t < 2 * RK * (kTS / 4); t += blockDim.x) {
+  for (int t = threadIdx.x; t < 2 * RK * (TS / 4); t += blockDim.x) {
     const int rk = t % RK, rem = t / RK;
     const int cy = rem & 1, cl = (rem >> 1) * 4;
     R q0[HK + 1], q1[HK + 1];                    // coefficients kc + 1 - i
@@ -274,9 +328,8 @@ __device__ __forceinline__ void idwt_tile(const R* __restrict__ llin, const R* _
   }
   __syncthreads();
   // columns: four adjacent output rows per thread likewise
-  static_assert(kTS * kTS == 4 * 256, "one group of four rows per thread");
-  {
-    const int cl = threadIdx.x % kTS, ml = (threadIdx.x / kTS) * 4;
+  for (int t = threadIdx.x; t < TS * (TS / 4); t += 256) {
+    const int cl = t % TS, ml = (t / TS) * 4;
     const int c = c0 + cl;
     const int km = (ml >> 1) + HK;
     R q0[HK + 1], q1[HK + 1];
