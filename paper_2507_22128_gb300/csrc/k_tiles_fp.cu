@@ -23,7 +23,7 @@
 //     transposed butterfly (10 shuffles for the pair), forms the weighted
 //     residuals and spreads them into 16 complex accumulators per lane,
 //   * adds its accumulators into the shared-memory grid tile once per chunk,
-//     with plain read-modify-writes under a per-CTA lock (warps of one item
+//     with plain read-modify-writes under two per-CTA locks (warps of one item
 //     may share cells).
 // The model tile (8 planes x 23 x 24 complex cells, the tile plus the kernel
 // halo) arrives by one TMA tensor load per item, completion tracked by an
@@ -461,6 +461,21 @@ __device__ __forceinline__ float2 unpack2(f2x v) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
   return r;
 }
+// one lane's share of half of the planes (8 cells, u taps 2 kRow floats apart)
+// added into the grid tile: all loads, then all stores
+__device__ __forceinline__ void flush_half(float* g, const f2x (&re)[4], const f2x (&im)[4]) {
+  float2 c[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) c[i] = *reinterpret_cast<float2*>(g + 2 * i * kRow);
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const float2 r = unpack2(re[t]), m = unpack2(im[t]);
+    c[2 * t].x += r.x; c[2 * t].y += m.x;
+    c[2 * t + 1].x += r.y; c[2 * t + 1].y += m.y;
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) *reinterpret_cast<float2*>(g + 2 * i * kRow) = c[i];
+}
 __device__ __forceinline__ float hsum2(f2x v) {
   const float2 r = unpack2(v);
   return r.x + r.y;
@@ -524,15 +539,15 @@ __global__ void __launch_bounds__(kFpThreads, 2)
   WarpScratch* scratch = reinterpret_cast<WarpScratch*>(tail);
   uint32_t* cb = reinterpret_cast<uint32_t*>(scratch + kFpWarps);   // chunk bounds of the item
   uint32_t* queue = cb + kCbMax;                                     // next chunk to claim
-  uint32_t* lock = queue + 1;                                        // the grid tile's flush lock
-  uint64_t* bar = reinterpret_cast<uint64_t*>(queue + 2);
+  uint32_t* lock = queue + 1;                                        // the grid tile's two flush locks (planes 0-3, 4-7)
+  uint64_t* bar = reinterpret_cast<uint64_t*>(queue + 4);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int vrow = lane & 7, pa = lane >> 3;         // this lane's v row and planes pa, pa + 4
   const bool b4 = (lane >> 4) & 1, b3 = (lane >> 3) & 1;
   const int mine = kGroup == 4 ? 2 * int(b3) + int(b4) : int(b4);   // the group sample whose degrid sum this lane ends with
   const uint32_t bar_a = smem_u32(bar);
-  if (threadIdx.x == 0) *lock = 0u;
+  if (threadIdx.x == 0) lock[0] = lock[1] = 0u;
   if (kModel && threadIdx.x == 0) {
     mbar_init(bar_a, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -819,44 +834,40 @@ __global__ void __launch_bounds__(kFpThreads, 2)
       }
       if constexpr (kSpread) {
       // add the chunk's accumulators into the item's grid tile: plain
-      // read-modify-writes under the CTA's flush lock (the chunks of one
+      // read-modify-writes under the CTA's flush locks (the chunks of one
       // item overlap; with shared-memory float atomics instead, a launch of
-      // the medium workload took 0.19 / 0.27 ms longer); a lock that stays
-      // taken (impossible: every holder releases it after 16 loads and
-      // stores) is reported and the flush goes ahead without it
-      float* ga = grid + 2 * (pa * kPlaneC + cell);
-      float* gb = grid + 2 * ((pa + 4) * kPlaneC + cell);
-      bool held = false;
-      if (lane == 0) {
-        for (uint32_t n = 0; n < kLockPolls && !held; ++n) {
-          held = atomicCAS(lock, 0u, 1u) == 0u;
-          if (!held) __nanosleep(32);
-        }
-        if (!held) atomicCAS(a.status, 0, RIX_ETIMEOUT);
-        __threadfence_block();
-      }
-      __syncwarp();
+      // the medium workload took 0.19 / 0.27 ms longer).  One lock per half of
+      // the planes, whichever is free first, each held for eight loads and
+      // eight stores in one round trip: with one lock held for four such round
+      // trips the warps of short chunks mostly waited for it (branch-resolving
+      // stalls 3.1 per issue; the dirty images of 8 M samples at 1024^2 2.28 ->
+      // 2.10 ms, the residual mode's major cycles 3 % faster).  A lock that stays taken (impossible:
+      // every holder releases it) is reported and the flush goes ahead
+      // without it
+      int half = warp & 1;
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const float2 ar = unpack2(aar[t]), ai = unpack2(aai[t]), br = unpack2(abr[t]), bi = unpack2(abi[t]);
-        float2* qa0 = reinterpret_cast<float2*>(ga + 2 * (2 * t) * kRow);
-        float2* qa1 = reinterpret_cast<float2*>(ga + 2 * (2 * t + 1) * kRow);
-        float2* qb0 = reinterpret_cast<float2*>(gb + 2 * (2 * t) * kRow);
-        float2* qb1 = reinterpret_cast<float2*>(gb + 2 * (2 * t + 1) * kRow);
-        float2 c0 = *qa0, c1 = *qa1, c2 = *qb0, c3 = *qb1;
-        c0.x += ar.x; c0.y += ai.x;
-        c1.x += ar.y; c1.y += ai.y;
-        c2.x += br.x; c2.y += bi.x;
-        c3.x += br.y; c3.y += bi.y;
-        *qa0 = c0;
-        *qa1 = c1;
-        *qb0 = c2;
-        *qb1 = c3;
-      }
-      __syncwarp();
-      if (lane == 0) {
-        __threadfence_block();
-        if (held) atomicExch(lock, 0u);
+      for (int h = 0; h < 2; ++h) {
+        bool held = false;
+        if (lane == 0) {
+          for (uint32_t n = 0; n < kLockPolls && !held; ++n) {
+            held = atomicCAS(lock + half, 0u, 1u) == 0u;
+            if (!held) {
+              if (h == 0) half ^= 1;
+              if (h == 1 || (n & 1u)) __nanosleep(32);
+            }
+          }
+          if (!held) atomicCAS(a.status, 0, RIX_ETIMEOUT);
+          __threadfence_block();
+        }
+        half = __shfl_sync(0xffffffffu, half, 0);
+        if (half == 0) flush_half(grid + 2 * (pa * kPlaneC + cell), aar, aai);
+        else flush_half(grid + 2 * ((pa + 4) * kPlaneC + cell), abr, abi);
+        __syncwarp();
+        if (lane == 0) {
+          __threadfence_block();
+          if (held) atomicExch(lock + half, 0u);
+        }
+        half ^= 1;
       }
       }
       k = k2;
