@@ -860,6 +860,7 @@ __global__ void __launch_bounds__(kFpThreads, 2)
           __threadfence_block();
         }
         half = __shfl_sync(0xffffffffu, half, 0);
+        __syncwarp();   // orders every lane's accesses after lane 0's acquire (a shuffle orders no memory)
         if (half == 0) flush_half(grid + 2 * (pa * kPlaneC + cell), aar, aai);
         else flush_half(grid + 2 * ((pa + 4) * kPlaneC + cell), abr, abi);
         __syncwarp();
