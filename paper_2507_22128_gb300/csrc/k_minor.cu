@@ -1033,7 +1033,9 @@ int op_msclean(Job* job, int p, const rix_msclean_params* prm, R* delta_out, cud
   }
 #undef RIX_CLEAN
   // at most four CTAs per SM: enough loads in flight for the sweeps, and
-  // every CTA reads every CTA's candidate at each iteration
+  // every CTA reads every CTA's candidate at each iteration.  The CTA's tile
+  // records (1.6 KB at 4096^2) stay below the shared memory a kernel has without
+  // an attribute: the attribute is the process's, and this size the job's
   const int ntiles = (n / ts) * (n / ts);
   int nblk = 0;
   size_t smem = 0;
@@ -1041,7 +1043,7 @@ int op_msclean(Job* job, int p, const rix_msclean_params* prm, R* delta_out, cud
     const int want = std::min(ctx->num_sms * per, ntiles);
     smem = (size_t)ceil_div(ntiles, want) * (sizeof(CleanTile<R>) + sizeof(int)) + 16;
     int per_sm = 0;
-    RIX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 32 * 1024) continue;
     RIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem));
     if (per_sm >= per || (int64_t)per_sm * ctx->num_sms >= want) nblk = want;
   }

@@ -26,3 +26,10 @@ def test_flush_locks_order_the_whole_warp():
     acquire, release = section[:first], section[last:]
     assert "__syncwarp()" in acquire[acquire.index("__threadfence_block()"):]
     assert "__threadfence_block()" in release[release.index("__syncwarp()"):]
+
+
+def test_clean_kernel_sets_no_attribute():
+    """A kernel's attributes belong to the process, and the shared memory of
+    k_msclean is sized by the job: a value set for one thread's launch would
+    bound another's."""
+    assert "cudaFuncSetAttribute" not in _source("k_minor.cu")
