@@ -11,6 +11,7 @@
 #include <cmath>
 #include <vector>
 
+#include "clean_bound.cuh"
 #include "rix_internal.cuh"
 #include "fft_device.cuh"
 #include "wavelet_device.cuh"
@@ -654,8 +655,7 @@ __global__ void __launch_bounds__(256) k_msclean(CleanArgs a) {
     }
     // a lower bound of the next peak
     const float fa = fabsf((float)amp) * 1.00001f;
-    const float keep = (float)Key::value(best.key) * (1.f - (float)a.gain) * 0.9999f;
-    float low = keep;
+    float low = clean_keep((float)Key::value(best.key), a.gain);
     if (b.key2 > 0) {
       const int y2 = b.pix2 / n, x2 = b.pix2 - (b.pix2 / n) * n;
       const float v2 = (float)Key::value(b.key2) * 0.9999f - fa * reach(best.s, (y2 / TS) * TS, (x2 / TS) * TS, best.pix).x;
