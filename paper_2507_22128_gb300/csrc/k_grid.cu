@@ -293,8 +293,6 @@ struct TileArgs {
   int slice, nsub;          // a work item is cut into nsub slices of `slice` entries (set_slices)
 };
 
-constexpr int kItemEntries = 2048;   // most entries of a work item (k_partition.cu)
-
 // How finely the work items are cut for `slots` resident CTAs.  A work item is
 // up to 2048 entries of one uv tile, so a small or centrally crowded
 // observation has a few long items and most SMs idle (19,841 samples at 128^2:

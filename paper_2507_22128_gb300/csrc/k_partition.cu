@@ -18,7 +18,6 @@ constexpr int kScanTile = kScanThreads * kScanItems;
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 16;
 constexpr int kSortTile = kSortThreads * kSortItems;  // 4096 keys per block
-constexpr int kChunk = 2048;                          // entries per gridder work item
 
 // ------------------------------------------------------------------ scan ----
 __global__ void __launch_bounds__(kScanThreads) k_scan_block(const uint32_t* __restrict__ in,
@@ -556,7 +555,7 @@ __global__ void k_seg_chunks(const uint32_t* __restrict__ starts, const uint32_t
   const uint32_t nseg = *nseg_p;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nseg; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t end = (i + 1 < nseg) ? starts[i + 1] : n;
-    chunks[i] = (uint32_t)((end - starts[i] + kChunk - 1) / kChunk);
+    chunks[i] = (uint32_t)((end - starts[i] + kItemEntries - 1) / kItemEntries);
   }
 }
 
@@ -565,7 +564,7 @@ __global__ void k_items(const uint32_t* __restrict__ starts, const uint32_t* __r
                         int64_t n, uint32_t* __restrict__ items, const uint32_t* __restrict__ nitems_p) {
   const uint32_t nseg = *nseg_p;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nseg; i += (int64_t)gridDim.x * blockDim.x) {
-    for (uint32_t c = 0; c < chunks[i]; ++c) items[coff[i] + c] = starts[i] + c * (uint32_t)kChunk;
+    for (uint32_t c = 0; c < chunks[i]; ++c) items[coff[i] + c] = starts[i] + c * (uint32_t)kItemEntries;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) items[*nitems_p] = (uint32_t)n;
 }

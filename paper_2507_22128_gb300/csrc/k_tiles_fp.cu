@@ -55,7 +55,6 @@ constexpr int kTileFloats = kW * kPlaneC * 2; // 8 planes
 constexpr int kTileBytes = kTileFloats * 4;   // 35,328 B (a multiple of 128)
 constexpr int kChunkMax = 32;                 // entries per batch (a warp's staging slot)
 constexpr int kChunkLimitMax = 256;           // most entries per chunk (the job's chunk limit)
-constexpr int kItemMax = 2048;                // entries per work item (the partition's item split)
 constexpr int kFpThreads = 256;
 constexpr int kFpWarps = kFpThreads / 32;
 constexpr uint32_t kWaitPolls = 1u << 24;     // bounded mbarrier wait
@@ -72,7 +71,7 @@ static_assert(kTileBytes % 128 == 0, "tile alignment");
 template <int BITS>
 struct TapOrder {
   static constexpr int kBins = 1 << BITS;
-  static constexpr int kRounds = kItemMax / 256;
+  static constexpr int kRounds = kItemEntries / 256;
   unsigned short cnt[8][kBins];
   unsigned short off[kBins];
   int wsum[8];
@@ -273,7 +272,7 @@ __global__ void k_psf_run_starts(const uint32_t* __restrict__ f, const uint32_t*
 }
 
 // The geometry and weight of every entry in key order, and the entries that
-// start a work item (the first of a run, and every kItemMax-th after it).
+// start a work item (the first of a run, and every kItemEntries-th after it).
 __global__ void k_psf_gather(const uint32_t* __restrict__ sv, const float4* __restrict__ geom_in,
                              const uint32_t* __restrict__ samples, const float* __restrict__ weight, int64_t e_begin,
                              const uint32_t* __restrict__ f, const uint32_t* __restrict__ ex,
@@ -284,7 +283,7 @@ __global__ void k_psf_gather(const uint32_t* __restrict__ sv, const float4* __re
     geom[i] = geom_in[src];
     w[i] = weight ? weight[samples[e_begin + src]] : 1.0f;
     const uint32_t run = ex[i] + f[i] - 1u;
-    iflag[i] = (((uint32_t)i - starts[run]) % (uint32_t)kItemMax) == 0u ? 1u : 0u;
+    iflag[i] = (((uint32_t)i - starts[run]) % (uint32_t)kItemEntries) == 0u ? 1u : 0u;
   }
 }
 
@@ -296,7 +295,7 @@ __global__ void k_psf_items(const uint32_t* __restrict__ iflag, const uint32_t* 
   if (blockIdx.x == 0 && threadIdx.x == 0) items[*n_items] = (uint32_t)n;
 }
 
-// Per work item (one PSF tile of one w-plane block, at most kItemMax entries;
+// Per work item (one PSF tile of one w-plane block, at most kItemEntries entries;
 // *n_items of them): the entries reordered stably by first tap, their unit
 // visibilities {w, 0, w, 0} written in that order, and the entries that
 // start a chunk (a new first tap, and every limit-th after) flagged.

@@ -108,6 +108,9 @@ template <typename C> __host__ __device__ __forceinline__ C cmulc(C a, C b) {  /
 constexpr double kC = 299792458.0;
 constexpr int kW = 8;            // ES kernel support (cells)
 constexpr double kBeta = 18.4;   // 2.30 * kW
+// most entries of a gridder work item (a run of sorted entries of one uv tile
+// and w-plane block): the partition cuts by it, the gridders size by it
+constexpr int kItemEntries = 2048;
 
 // ---------------------------------------------------------------------------
 // gridder building blocks shared by k_grid.cu and k_tiles_fp.cu

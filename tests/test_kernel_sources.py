@@ -33,3 +33,11 @@ def test_clean_kernel_sets_no_attribute():
     k_msclean is sized by the job: a value set for one thread's launch would
     bound another's."""
     assert "cudaFuncSetAttribute" not in _source("k_minor.cu")
+
+
+def test_one_size_of_a_work_item():
+    """The partition cuts work items, and the gridders walk, order and slice them,
+    by the same number."""
+    found = [(f, line.strip()) for f in sorted(os.listdir(CSRC)) for line in _source(f).splitlines()
+             if re.search(r"constexpr\s+int\s+k\w*\s*=\s*2048\b", line)]
+    assert len(found) == 1 and found[0][0] == "rix_internal.cuh", found
