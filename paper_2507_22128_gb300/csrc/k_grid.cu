@@ -289,23 +289,15 @@ struct TileArgs {
   const void* geom;         // EntryGeom<R> per sorted entry, from entry geom_off on
   int64_t geom_off;
   int64_t ent_begin, ent_count;   // the partition's entries
+  int64_t max_tile;         // ... of its fullest uv tile
   int* status;              // the job's status word (RIX_EINTERNAL on a failed check)
   int slice, nsub;          // a work item is cut into nsub slices of `slice` entries (set_slices)
 };
 
-// How finely the work items are cut for `slots` resident CTAs.  A work item is
-// up to 2048 entries of one uv tile, so a small or centrally crowded
-// observation has a few long items and most SMs idle (19,841 samples at 128^2:
-// 207 us per gridding launch and 31 us per degridding, the time of one full
-// item; 17 and 5 us cut).  A slice is at most a quarter of a slot's share of
-// the entries, a power of two of at least 64: each slice stages and flushes
-// its tile, about the work of ten entries.
-void set_slices(TileArgs& a, int64_t slots) {
-  const int64_t share = a.ent_count / (4 * std::max<int64_t>(slots, 1));
-  int slice = 64;
-  while (slice < kItemEntries && slice < share) slice *= 2;
-  a.slice = slice;
-  a.nsub = kItemEntries / slice;
+// `sums`: the launch adds into the grid in FP32 (slice_entries)
+void set_slices(TileArgs& a, int64_t slots, bool sums) {
+  a.slice = slice_entries(a.ent_count, slots, sums ? a.max_tile : 0);
+  a.nsub = kItemEntries / a.slice;
 }
 
 // On the PSF's 2N grid (x_psf = 2 x exactly), an image-grid tile of side T
@@ -562,7 +554,7 @@ int launch_tiles_impl(const Ctx* ctx, TileArgs a, cudaStream_t st) {
   RIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, sm));
   per_sm = std::max(per_sm, 1);
   const int64_t slots = (int64_t)ctx->num_sms * per_sm;
-  set_slices(a, slots);
+  set_slices(a, slots, kUseGrid && sizeof(R) == 4);
   const int64_t blocks = std::min<int64_t>(a.item_count * a.nsub, slots);
   if (blocks <= 0) return RIX_OK;
   timing_mark(kTimeTiles, st, true);
@@ -791,7 +783,7 @@ int launch_tiles_ws(const Ctx* ctx, TileArgs a, cudaStream_t st) {
   RIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, sm));
   per_sm = std::max(per_sm, 1);
   const int64_t slots = (int64_t)ctx->num_sms * per_sm;
-  set_slices(a, slots);
+  set_slices(a, slots, sizeof(R) == 4);
   const int64_t blocks = std::min<int64_t>(a.item_count * a.nsub, slots);
   if (blocks <= 0) return RIX_OK;
   timing_mark(kTimeTiles, st, true);
@@ -847,6 +839,7 @@ TileArgs base_args(const Job* job, const Part& pt) {
   a.geom_off = 0;
   a.ent_begin = pt.ent_begin;
   a.ent_count = pt.ent_count;
+  a.max_tile = pt.max_tile;
   a.status = job->status.as<int>();
   return a;
 }

@@ -550,12 +550,16 @@ __global__ void k_seg_starts(const uint32_t* __restrict__ f, const uint32_t* __r
     if (f[e]) starts[ex[e]] = (uint32_t)e;
 }
 
+// work items per segment (the entries of one key), and each partition's longest
+// segment (the partition is the key from bit `pshift` on)
 __global__ void k_seg_chunks(const uint32_t* __restrict__ starts, const uint32_t* __restrict__ nseg_p,
-                             int64_t n, uint32_t* __restrict__ chunks) {
+                             int64_t n, const uint32_t* __restrict__ keys, int pshift,
+                             uint32_t* __restrict__ chunks, uint32_t* __restrict__ longest) {
   const uint32_t nseg = *nseg_p;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nseg; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t end = (i + 1 < nseg) ? starts[i + 1] : n;
     chunks[i] = (uint32_t)((end - starts[i] + kItemEntries - 1) / kItemEntries);
+    atomicMax(&longest[(uint64_t)keys[starts[i]] >> pshift], (uint32_t)(end - starts[i]));
   }
 }
 
@@ -672,6 +676,7 @@ int partition_job(Job* job, const double* uvw, int64_t nrow, const float* weight
     double ells[kMaxPart];
     int win[kMaxPart * 4];
     uint32_t totals[4];
+    uint32_t longest[kMaxPart];   // entries of the fullest tile (of one w-plane block)
     int64_t ent_begin[kMaxPart + 1];
     int64_t item_range[kMaxPart + 1];
   };
@@ -835,7 +840,8 @@ int partition_job(Job* job, const double* uvw, int64_t nrow, const float* weight
     uint32_t* starts = wa;
     ::rix::note_launch(); k_seg_starts<<<eb, 256, 0, st>>>(kt, vt, n_ent, starts);
     uint32_t* chunks = wb;
-    ::rix::note_launch(); k_seg_chunks<<<eb, 256, 0, st>>>(starts, &sm_d->totals[1], n_ent, chunks);
+    ::rix::note_launch(); k_seg_chunks<<<eb, 256, 0, st>>>(starts, &sm_d->totals[1], n_ent, job->keys.as<uint32_t>(),
+                                                             2 * kl.bt + kl.bw, chunks, sm_d->longest);
     // chunk offsets into kt (flags no longer needed)
     uint32_t nseg_h = 0;
     RIX_CUDA(cudaMemcpyAsync(&nseg_h, &sm_d->totals[1], sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
@@ -891,6 +897,7 @@ int partition_job(Job* job, const double* uvw, int64_t nrow, const float* weight
     pt.item_begin = sm_h.item_range[p];
     pt.item_count = sm_h.item_range[p + 1] - sm_h.item_range[p];
     pt.wsum = sm_h.wsum[p];
+    pt.max_tile = sm_h.longest[p];
     S.part_count[p] = pt.ent_count;
     S.part_weight[p] = pt.wsum;
     if (pt.ent_count > 0) {

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/rix.h"
+#include "slice_rule.cuh"
 
 namespace rix {
 
@@ -108,9 +109,6 @@ template <typename C> __host__ __device__ __forceinline__ C cmulc(C a, C b) {  /
 constexpr double kC = 299792458.0;
 constexpr int kW = 8;            // ES kernel support (cells)
 constexpr double kBeta = 18.4;   // 2.30 * kW
-// most entries of a gridder work item (a run of sorted entries of one uv tile
-// and w-plane block): the partition cuts by it, the gridders size by it
-constexpr int kItemEntries = 2048;
 
 // ---------------------------------------------------------------------------
 // gridder building blocks shared by k_grid.cu and k_tiles_fp.cu
@@ -286,6 +284,7 @@ constexpr int kMaxScales = 8;
 struct Part {
   int64_t ent_begin = 0, ent_count = 0;     // range in the sorted entries
   int64_t item_begin = 0, item_count = 0;   // range in the work items
+  int64_t max_tile = 0;                     // entries of the fullest uv tile (of one w-plane block)
   double wsum = 0.0;
   int win_lo = 0, win_n = 0;                // uv window on the 2N grid
   int pwin_lo = 0, pwin_n = 0;              // uv window on the 4N PSF grid
