@@ -895,6 +895,18 @@ int check_geom(const XformGeom& g) {
   return RIX_OK;
 }
 
+// ... and, for a row pass, the tables its pixel factors come from: the screen
+// table, or corr with n - 1 in the form that the pass reads
+template <typename R>
+int check_rows(const XformGeom& g, bool inverse) {
+  RIX_TRY(check_geom<R>(g));
+  if (g.mode == kFacNone || (g.mode == kFacPhase && g.screen)) return RIX_OK;
+  const bool pairs = sizeof(R) == 4 && inverse && g.M != g.L;
+  if (!g.corr || (g.mode == kFacPhase && (pairs ? !g.nm1f : !g.nm1)))
+    return set_error(RIX_EINVAL, "transform rows without their factor tables");
+  return RIX_OK;
+}
+
 // calls f(LOGF) with the transform length's log2 as a compile-time constant
 template <int LO, int HI, class Fn>
 int with_log(int logf, const Fn& f) {

@@ -9,7 +9,7 @@ namespace rix {
 
 template <typename R>
 int fwd_rows(const Ctx* ctx, const XformGeom& g, const R* img, cplx<R>* T, cudaStream_t st) {
-  RIX_TRY(check_geom<R>(g));
+  RIX_TRY(check_rows<R>(g, false));
   if constexpr (sizeof(R) == 4) {
     if (g.M != g.L)
       return with_log<kMinLogF + 1, kMaxLogL<R>>(g.logL, [&](auto ll) {
@@ -65,7 +65,7 @@ int inv_rows_groups(const Ctx* ctx, const XformGeom& g, int max_groups) {
 template <typename R>
 int inv_rows(const Ctx* ctx, const XformGeom& g0, const cplx<R>* T, R* img, double scale, int accumulate,
              cudaStream_t st, R* group_buf, int max_groups) {
-  RIX_TRY(check_geom<R>(g0));
+  RIX_TRY(check_rows<R>(g0, true));
   XformGeom g = g0;
   const int P = g.nplanes;
   const int G = inv_rows_groups<R>(ctx, g, max_groups < 0 ? 16 : max_groups);

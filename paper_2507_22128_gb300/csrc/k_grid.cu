@@ -855,8 +855,8 @@ XformGeom plane_geom(const Job* job, const Part& pt, bool psf) {
   g.nplanes = job->nw > 0 ? job->nw : 1;
   g.mode = job->nw > 0 ? kFacPhase : kFacReal;
   g.corr = psf ? job->corr_psf.p : job->corr_img.p;
-  g.nm1 = psf ? job->nm1_psf.as<double>() : job->nm1_img.as<double>();
   if (psf && !job->fp64) g.nm1f = job->nm1_psf.as<float2>();
+  else g.nm1 = psf ? job->nm1_psf.as<double>() : job->nm1_img.as<double>();
   g.w0 = job->stats.w_min - 0.5 * job->ww * job->stats.dw;
   g.dw = job->stats.dw;
   // the image grid's factors are tabulated once per job (the PSF's grid is
@@ -1058,8 +1058,8 @@ int op_psf_tiled(Job* job, int p, cudaStream_t st) {
     if (ws) {
       if ((rc = fill_correction<R>(job, n, job->ng, ox, oy, n, corr, nm1, sizeof(R) == 4, st)) != RIX_OK) break;
       g.corr = corr;
-      g.nm1 = nm1;
-      if (sizeof(R) == 4) g.nm1f = reinterpret_cast<const float2*>(nm1);
+      g.nm1 = sizeof(R) == 4 ? nullptr : nm1;
+      g.nm1f = sizeof(R) == 4 ? reinterpret_cast<const float2*>(nm1) : nullptr;
     }
     if (cudaMemsetAsync(pt.resid_planes.p, 0, (size_t)np * pt.win_n * pt.win_n * sizeof(cplx<R>), st) != cudaSuccess) {
       rc = set_error(RIX_ECUDA, "memset");

@@ -188,8 +188,10 @@ struct XformGeom {
   int nplanes;
   int mode;                    // FactorMode
   const void* corr;            // Real [M][M] or null
-  const double* nm1;           // double [M][M]: n - 1 per pixel (kFacPhase)
-  const float2* nm1f = nullptr;   // FP32 inverse rows without a screen table: n - 1 as pairs of floats
+  // n - 1 per pixel (kFacPhase without a screen table), [M][M]: one table, as
+  // doubles, or as pairs of floats for the FP32 inverse rows of padded planes
+  const double* nm1;
+  const float2* nm1f = nullptr;
   double w0, dw;               // plane p sits at w0 + p * dw (kFacPhase)
   int herm = 0;                // inverse rows: complete columns [S, L) by conjugate symmetry (lo = 0)
   // kFacPhase, optional: cplx [nplanes][M][M] of corr * exp(-2 pi i w_p (n-1)),
@@ -354,7 +356,8 @@ struct Job {
   int bt = 0, bw = 0, bp = 0;
   // corrections
   DevBuf corr_img, corr_psf;                // Real [N][N], [2N][2N]
-  DevBuf nm1_img, nm1_psf;                  // n - 1 per pixel (w-stacked): double; the PSF's in FP32 jobs a pair of floats
+  DevBuf nm1_img;                           // n - 1 per pixel (w-stacked): double
+  DevBuf nm1_psf;                           // ... the PSF's: double, in FP32 jobs float2 (high, low)
   DevBuf screen_img;                        // w-stacked: corr x phase screen per plane, image grid
   DevBuf gam;                               // Real [P][2N][2N] filters (u-major spectra)
   Part part[kMaxPart];
