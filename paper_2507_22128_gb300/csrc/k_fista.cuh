@@ -717,20 +717,25 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 && LOGL <= 12 ? 2 
   fista_iterations<R, LOGL, DICT>(a, a.f, a.nb, (int)blockIdx.x, (int)gridDim.x, [&] { return grid_barrier(bar); });
 }
 
-// Small images: a cluster of kClusterCtas CTAs per loop, joined by the cluster
+// Small images: a cluster of up to kClusterCtas CTAs per loop, joined by the cluster
 // barrier, instead of the whole grid by a counter in global memory.  A phase of
 // a 128 x 128 loop has 4 to 16 units, so 16 CTAs run it as fast as 152 do, and
 // the barrier, a few hundred nanoseconds instead of one to two microseconds of
 // atomics and polling, was most of its time (50 iterations of both partitions
 // at 128^2: 1.73 -> 1.28 ms against the dataflow schedule of the batch).
+// 16 CTAs is above the size that every device takes (8): a device, or a part of
+// one, that cannot place such a cluster runs the loop on the largest that it can,
+// in an instance of its own (CTAS = 0: the launch's size; with it in every launch
+// the phases' loops are loops again, 7.50 -> 7.57 ms for the 128 x 128 job).
 constexpr int kClusterCtas = 16;
 constexpr int kClusterLogL = 8;   // longest transform 2N that takes this path
 
-template <typename R, int LOGL, int DICT>
+template <typename R, int LOGL, int DICT, int CTAS>
 __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 2 : 1)
     k_fista_cluster(const __grid_constant__ FistaArgs<R> a) {
-  const int b = (int)blockIdx.x / kClusterCtas, rank = (int)blockIdx.x % kClusterCtas;
-  fista_iterations<R, LOGL, DICT>(a, a.f + b, 1, rank, kClusterCtas, [] {
+  const int ctas = CTAS > 0 ? CTAS : (int)gridDim.x / a.nb;   // the cluster's
+  const int b = (int)blockIdx.x / ctas, rank = (int)blockIdx.x % ctas;
+  fista_iterations<R, LOGL, DICT>(a, a.f + b, 1, rank, ctas, [] {
     // every thread of the cluster arrives (releasing its writes) and waits
     // (acquiring the others'): a hardware barrier, which completes because
     // every CTA of the cluster runs the same phases
@@ -911,6 +916,18 @@ double mom_host(int iters, R* mom) {
   return t;
 }
 
+// launch(ctas) with the largest cluster that it takes: kClusterCtas CTAs, then
+// half as many down to one while the launch is refused; the last one's result
+template <class Launch>
+cudaError_t launch_clusters(const Launch& launch) {
+  cudaError_t e = cudaSuccess;
+  for (int c = kClusterCtas; c >= 1; c /= 2) {
+    if ((e = launch(c)) == cudaSuccess) break;
+    if (c > 1) cudaGetLastError();
+  }
+  return e;
+}
+
 template <typename R, int LOGL, int DICT>
 int launch_fista_loop(const Ctx* ctx, const FistaLoop<R>* f, int nb, cudaStream_t st) {
   using F = FistaShape<R, LOGL, DICT>;
@@ -933,15 +950,10 @@ int launch_fista_loop(const Ctx* ctx, const FistaLoop<R>* f, int nb, cudaStream_
   }
   args.t_tab = mom_host<R>(std::min(f[0].iters, kMomTab), args.mom_tab);
   if constexpr (LOGL <= kClusterLogL) {
-    auto ck = k_fista_cluster<R, LOGL, DICT>;
-    RIX_CUDA(cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    RIX_CUDA(cudaFuncSetAttribute(ck, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = kClusterCtas;
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(nb * kClusterCtas));
     cfg.blockDim = dim3(kFftThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -949,7 +961,15 @@ int launch_fista_loop(const Ctx* ctx, const FistaLoop<R>* f, int nb, cudaStream_
     cfg.numAttrs = 1;
     ::rix::note_launch();
     timing_mark(kTimeMinorLoop, st, true);
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, ck, args);
+    const cudaError_t e = launch_clusters([&](int ctas) {
+      attr.val.clusterDim.x = (unsigned)ctas;
+      cfg.gridDim = dim3((unsigned)(nb * ctas));
+      auto ck = ctas == kClusterCtas ? k_fista_cluster<R, LOGL, DICT, kClusterCtas> : k_fista_cluster<R, LOGL, DICT, 0>;
+      cudaError_t e = cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e == cudaSuccess && ctas == kClusterCtas)
+        e = cudaFuncSetAttribute(ck, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, ck, args) : e;
+    });
     timing_mark(kTimeMinorLoop, st, false);
     if (e != cudaSuccess) return set_error(RIX_ECUDA, "FISTA loop launch: %s", cudaGetErrorString(e));
     return RIX_OK;
