@@ -916,6 +916,19 @@ double mom_host(int iters, R* mom) {
   return t;
 }
 
+// CTAs per SM of the loops on the whole grid: two for a batch of loops, one for a
+// single loop, so that another partition's or job's fits beside it.  Two as well
+// for the loop of an unpartitioned job with the concatenated dictionary from
+// 1024^2 on, where one CTA per SM leaves most of its phases waiting: 50 iterations
+// of one / two / three jobs in flight, one CTA against two, 17.5 / 37.3 / 39.3
+// against 12.5 / 24.1 / 36.6 ms (2048^2: 56 / 120 / 135, 38 / 76 / 121).  Not below
+// (512^2, one / two / four jobs: 5.8 / 9.0 / 16.9 against 6.2 / 11.2 / 21.5), and
+// not with Db4, which gains only while no other job runs (1024^2, one / two: 3.2 /
+// 4.3 against 2.6 / 5.1; 512^2: 1.7 / 2.1 against 2.0 / 4.0).
+constexpr int loop_ctas_per_sm(int nb, bool solo, int dict, int n) {
+  return nb > 1 || (solo && dict != RIX_DICT_DB4 && n >= 1024) ? 2 : 1;
+}
+
 // launch(ctas) with the largest cluster that it takes: kClusterCtas CTAs, then
 // half as many down to one while the launch is refused; the last one's result
 template <class Launch>
@@ -979,10 +992,7 @@ int launch_fista_loop(const Ctx* ctx, const FistaLoop<R>* f, int nb, cudaStream_
     int per_sm = 0;
     RIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFftThreads, smem));
     if (per_sm < 1) return set_error(RIX_EINVAL, "FISTA loop does not fit on an SM (%zu B shared)", smem);
-    // two CTAs per SM for a batch of loops or the loop of an unpartitioned job (50
-    // iterations at 1024^2 3.34 -> 2.52 ms); one for a single partition's loop, so
-    // that another partition's fits beside it
-    const int nblk = ctx->num_sms * std::min(per_sm, nb > 1 || f[0].solo ? 2 : 1);
+    const int nblk = ctx->num_sms * std::min(per_sm, loop_ctas_per_sm(nb, f[0].solo, DICT, F::N));
     if constexpr (DICT == RIX_DICT_DB4) {
       if (nb > 1) {
         // several loops (Db4): the dataflow schedule instead of grid barriers
