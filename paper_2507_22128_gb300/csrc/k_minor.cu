@@ -397,13 +397,54 @@ __device__ __forceinline__ R clean_scale(const CleanArgs& a, R peak, int s) {
   return peak != R(0) ? (R)a.bias[s] / peak : R(0);
 }
 
+// component `it` of the list, by CTA 0: recorded, and its scale function added to
+// the model image, clipped to it
+template <typename R>
+__device__ __forceinline__ void add_component(const CleanArgs& a, int it, int s, int pix, R amp) {
+  if (threadIdx.x == 0) {
+    a.comp_s[it] = s;
+    a.comp_pix[it] = pix;
+    a.comp_amp[it] = (double)amp;
+  }
+  const int n = a.n, py = pix / n, px = pix - py * n;
+  const int rad = a.st_rad[s], w = 2 * rad + 1;
+  const R* stn = static_cast<const R*>(a.stencil) + a.st_off[s];
+  R* model = static_cast<R*>(a.model);
+  for (int k = threadIdx.x; k < w * w; k += blockDim.x) {
+    const int dy = k / w - rad, dx = k % w - rad;
+    const int yy = py + dy, xx = px + dx;
+    if (yy >= 0 && yy < n && xx >= 0 && xx < n) model[(int64_t)yy * n + xx] += amp * stn[k];
+  }
+}
+
+// value v of scale s at pixel pix taken into the running candidate c (a value
+// that is not a number is no candidate and no maximum)
+template <typename R>
+__device__ __forceinline__ void take_candidate(Cand<R>& c, R v, R scl, int s, int pix, int allowed) {
+  using Key = OrdKey<R>;
+  const typename Key::K ak = Key::of_abs(v);
+  if (s == 0 && ak > c.r0max && ak <= Key::kInf) c.r0max = ak;
+  if ((allowed >> s) & 1) {
+    const typename Key::K key = Key::of(fabs(v) * scl);
+    if (key >= c.key && key <= Key::kInf && (key > c.key || s < c.s || (s == c.s && pix < c.pix))) {
+      c.key = key;
+      c.rval = v;
+      c.s = s;
+      c.pix = pix;
+    }
+  }
+}
+
+constexpr int kCleanTile = 32;   // TS: side of a lazily updated tile
+
 // How far a component of scale sc moves the candidates of a TS x TS block of
 // the (2n)^2 grid of relative positions, per unit amplitude: x = the largest
 // |P_{s,sc}| b_s / P_ss(0) over the allowed scales, y = the largest |P_{0,sc}|
 // (rounded up; infinite where a value is not finite), [ns][2n / TS][2n / TS].
 // One warp per block.
-template <typename R, int TS>
+template <typename R>
 __global__ void __launch_bounds__(256) k_clean_reach(CleanArgs a, float2* __restrict__ out) {
+  constexpr int TS = kCleanTile;
   const int n2 = 2 * a.n, nb = n2 / TS, ns = a.ns;
   const int64_t n2sq = (int64_t)n2 * n2, blocks = (int64_t)ns * nb * nb;
   const R* P = static_cast<const R*>(a.P);
@@ -478,26 +519,26 @@ struct CleanTile {
 };
 
 // iterations between two updates of every tile: at 2048^2 FP32 26.1 / 26.7 us
-// per iteration with 8 / 16 (30.3 with 4), at 512^2 FP64 13.0 / 15.1 (12.1 with 4)
+// per iteration with 8 / 16 (30.3 with 4)
 constexpr int kCleanSweep = 8;
 
-// The whole minor cycle in one cooperative launch.  The components are those
-// of updating every scale residual at every iteration, and every residual
-// value goes through the same subtractions in the same order, but a tile is
-// updated only when it could hold the next peak: its last exact maximum plus
-// the reach of the components since (k_clean_reach) is compared with a lower
-// bound of the next peak, the larger of the cleaned peak's remainder and the
-// runner-up's value less the new component's reach there.  All tiles catch up
-// every kCleanSweep iterations, so the work stays even and the residuals are
-// read and written once per sweep instead of once per component: at 2048^2
-// with four scales 43 -> 26 us per iteration (201 MB moved by each before), at
-// 512^2 in FP64 with three 25 -> 13 us (the integer comparisons included).  The stopping rule needs max |R_0| < threshold exactly: a CTA none
-// of whose tiles is surely above it updates those that could be.
+// The whole minor cycle in one cooperative launch, on large images.  The
+// components are those of updating every scale residual at every iteration
+// (k_msclean_sweep), and every residual value goes through the same subtractions
+// in the same order, but a tile is updated only when it could hold the next peak:
+// its last exact maximum plus the reach of the components since (k_clean_reach) is
+// compared with a lower bound of the next peak, the larger of the cleaned peak's
+// remainder and the runner-up's value less the new component's reach there.  All
+// tiles catch up every kCleanSweep iterations, so the work stays even and the
+// residuals are read and written once per sweep instead of once per component.
+// The stopping rule needs max |R_0| < threshold exactly: a CTA none of whose
+// tiles is surely above it updates those that could be.
 // One bounded grid barrier per iteration separates the updates from the
 // selection (double-buffered slots); a barrier that gives up (RIX_ETIMEOUT in
 // the status word) ends every CTA.  NS = the number of scales.
-template <typename R, int NS, int TS>
+template <typename R, int NS>
 __global__ void __launch_bounds__(256) k_msclean(CleanArgs a) {
+  constexpr int TS = kCleanTile;
   using Key = OrdKey<R>;
   constexpr int PX = TS * TS / 256;
   GridBarrier bar{a.barrier, a.status, 0u};
@@ -561,18 +602,7 @@ __global__ void __launch_bounds__(256) k_msclean(CleanArgs a) {
 #pragma unroll
       for (int s = 0; s < NS; ++s) {
         if (upto > from) Rs[s * npix + pix] = v[k][s];
-        // (a NaN is no candidate and no maximum)
-        const typename Key::K ak = Key::of_abs(v[k][s]);
-        if (s == 0 && ak > c.r0max && ak <= Key::kInf) c.r0max = ak;
-        if ((a.allowed >> s) & 1) {
-          const typename Key::K key = Key::of(fabs(v[k][s]) * scl[s]);
-          if (key >= c.key && key <= Key::kInf && (key > c.key || s < c.s || (s == c.s && pix < c.pix))) {
-            c.key = key;
-            c.rval = v[k][s];
-            c.s = s;
-            c.pix = pix;
-          }
-        }
+        take_candidate<R>(c, v[k][s], scl[s], s, pix, a.allowed);
       }
     }
     c = block_reduce(c, sh);
@@ -636,23 +666,7 @@ __global__ void __launch_bounds__(256) k_msclean(CleanArgs a) {
     const Cand<R> best = b.c;
     if (it >= a.niter || Key::value(best.r0max) < (R)a.threshold || best.key < 0 || peak[best.s] == R(0)) break;
     const R amp = (R)a.gain * best.rval / peak[best.s];
-    const int py = best.pix / n, px = best.pix - py * n;
-    if (blockIdx.x == 0) {
-      if (threadIdx.x == 0) {
-        a.comp_s[it] = best.s;
-        a.comp_pix[it] = best.pix;
-        a.comp_amp[it] = (double)amp;
-      }
-      // model += amp * B_s(. - p*), clipped to the image
-      const int rad = a.st_rad[best.s], w = 2 * rad + 1;
-      const R* stn = static_cast<const R*>(a.stencil) + a.st_off[best.s];
-      R* model = static_cast<R*>(a.model);
-      for (int k = threadIdx.x; k < w * w; k += blockDim.x) {
-        const int dy = k / w - rad, dx = k % w - rad;
-        const int yy = py + dy, xx = px + dx;
-        if (yy >= 0 && yy < n && xx >= 0 && xx < n) model[(int64_t)yy * n + xx] += amp * stn[k];
-      }
-    }
+    if (blockIdx.x == 0) add_component<R>(a, it, best.s, best.pix, amp);
     // a lower bound of the next peak
     const float fa = fabsf((float)amp) * 1.00001f;
     float low = clean_keep((float)Key::value(best.key), a.gain);
@@ -678,6 +692,78 @@ __global__ void __launch_bounds__(256) k_msclean(CleanArgs a) {
       if (hot[i] || (!above && !((tile[i].r0 + tile[i].grow0) * 1.0001f < thr * 0.9999f)))
         update(i, it + 1, best.s, best.pix, amp);
     publish(it + 1);
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *a.count = it;
+}
+
+// The same minor cycle with every residual updated at every iteration: the sweep
+// that subtracts a component finds the next peak.  The registers of four CTAs per
+// SM, so that a pixel's loads of all scales are in flight together (four scales at
+// 1024^2 14.7 us per iteration with the 40 registers the compiler takes by itself,
+// 12.8 with these).
+template <typename R, int NS>
+__global__ void __launch_bounds__(256, sizeof(R) == 8 && NS > 6 ? 3 : 4) k_msclean_sweep(CleanArgs a) {
+  using Key = OrdKey<R>;
+  GridBarrier bar{a.barrier, a.status, 0u};
+  __shared__ Cand<R> sh[32];
+  const int n = a.n, n2 = 2 * a.n;
+  const int64_t npix = (int64_t)n * n;
+  R* __restrict__ Rs = static_cast<R*>(a.R);
+  const R* __restrict__ P = static_cast<const R*>(a.P);
+  Cand<R>* slots = static_cast<Cand<R>*>(a.slots);
+  __shared__ R peak[kMaxScales], scl[kMaxScales];
+  if (threadIdx.x < NS) {
+    const int s = threadIdx.x;
+    peak[s] = P[((int64_t)(s * NS + s) * n2 + n) * n2 + n];
+    scl[s] = clean_scale<R>(a, peak[s], s);
+  }
+  __syncthreads();
+  const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
+  const int logn = 31 - __clz(n);   // n is a power of two
+  const int64_t n2sq = (int64_t)n2 * n2;
+  // sweep with the subtraction of component (sc, py, px, amp) (amp = 0: none)
+  auto sweep = [&](int sc, int py, int px, R amp) {
+    Cand<R> c = no_cand<R>();
+    const R* __restrict__ psc = P + (int64_t)sc * n2sq;   // P_{s, sc} = psc + s NS (2n)^2
+    for (int64_t i = gtid; i < npix; i += gstride) {
+      const int y = (int)(i >> logn), x = (int)(i & (n - 1));
+      // P_{s,sc}(y - py, x - px) on the centred 2n grid
+      const int64_t pp = (int64_t)(n + y - py) * n2 + (n + x - px);
+      R v[NS];
+#pragma unroll
+      for (int s = 0; s < NS; ++s) v[s] = Rs[s * npix + i];
+      if (amp != R(0)) {
+        R q[NS];
+#pragma unroll
+        for (int s = 0; s < NS; ++s) q[s] = psc[(int64_t)s * NS * n2sq + pp];
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+          v[s] -= amp * q[s];
+          Rs[s * npix + i] = v[s];
+        }
+      }
+#pragma unroll
+      for (int s = 0; s < NS; ++s) take_candidate<R>(c, v[s], scl[s], s, (int)i, a.allowed);
+    }
+    return block_reduce(c, sh);
+  };
+
+  Cand<R> loc = sweep(0, 0, 0, R(0));
+  if (threadIdx.x == 0) slots[blockIdx.x] = loc;
+  int it = 0;
+  for (;; ++it) {
+    if (!grid_barrier(bar)) return;
+    const Cand<R>* cur = slots + (int64_t)(it & 1) * gridDim.x;
+    Cand<R> c = no_cand<R>();
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) c = merge(c, cur[b]);
+    const Cand<R> best = block_reduce(c, sh);
+    if (it >= a.niter || Key::value(best.r0max) < (R)a.threshold || best.key < 0 || peak[best.s] == R(0)) break;
+    const R amp = (R)a.gain * best.rval / peak[best.s];
+    const int py = best.pix / n, px = best.pix - py * n;
+    if (blockIdx.x == 0) add_component<R>(a, it, best.s, best.pix, amp);
+    loc = sweep(best.s, py, px, amp);
+    if (threadIdx.x == 0) slots[(int64_t)((it + 1) & 1) * gridDim.x + blockIdx.x] = loc;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) *a.count = it;
 }
@@ -1022,26 +1108,26 @@ int op_msclean(Job* job, int p, const rix_msclean_params* prm, R* delta_out, cud
   }
   // state: delta image, components, slots
   const int cap = std::max(prm->niter, 1);
-  // 32 x 32 tiles, 16 x 16 for small images (a tile per CTA down to 64^2)
-  const int ts = n >= 512 ? 32 : 16;
+  const bool lazy = clean_lazy(sizeof(R) == 8, n, ns);
+  constexpr int ts = kCleanTile;
   void (*kern)(CleanArgs) = nullptr;
 #define RIX_CLEAN(NS) \
-  case NS: kern = ts == 32 ? k_msclean<R, NS, 32> : k_msclean<R, NS, 16>; break;
+  case NS: kern = lazy ? k_msclean<R, NS> : k_msclean_sweep<R, NS>; break;
   switch (ns) {
     RIX_CLEAN(1) RIX_CLEAN(2) RIX_CLEAN(3) RIX_CLEAN(4) RIX_CLEAN(5) RIX_CLEAN(6) RIX_CLEAN(7) RIX_CLEAN(8)
     default: return set_error(RIX_EINVAL, "%d scales", ns);
   }
 #undef RIX_CLEAN
-  // at most four CTAs per SM: enough loads in flight for the sweeps, and
-  // every CTA reads every CTA's candidate at each iteration.  The CTA's tile
-  // records (1.6 KB at 4096^2) stay below the shared memory a kernel has without
-  // an attribute: the attribute is the process's, and this size the job's
-  const int ntiles = (n / ts) * (n / ts);
+  // every CTA reads every CTA's candidate at each iteration: no more of them than
+  // clean_ctas_per_sm.  The CTA's tile records (1.6 KB at 4096^2) stay below the
+  // shared memory a kernel has without an attribute: the attribute is the
+  // process's, and this size the job's
+  const int units = lazy ? (n / ts) * (n / ts) : (int)ceil_div(npix, 256);   // tiles, or CTAs with a pixel per thread
   int nblk = 0;
   size_t smem = 0;
-  for (int per = 4; per >= 1 && nblk == 0; --per) {
-    const int want = std::min(ctx->num_sms * per, ntiles);
-    smem = (size_t)ceil_div(ntiles, want) * (sizeof(CleanTile<R>) + sizeof(int)) + 16;
+  for (int per = clean_ctas_per_sm(sizeof(R) == 8, n, ns, lazy); per >= 1 && nblk == 0; --per) {
+    const int want = std::min(ctx->num_sms * per, units);
+    if (lazy) smem = (size_t)ceil_div(units, want) * (sizeof(CleanTile<R>) + sizeof(int)) + 16;
     int per_sm = 0;
     if (smem > 32 * 1024) continue;
     RIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem));
@@ -1050,7 +1136,8 @@ int op_msclean(Job* job, int p, const rix_msclean_params* prm, R* delta_out, cud
   if (nblk == 0) return set_error(RIX_EINVAL, "ms-CLEAN kernel does not fit on an SM");
   const size_t comp_bytes = (size_t)cap * (2 * sizeof(int) + sizeof(double)) + 16;
   RIX_TRY(ensure<R>(job, pt.ms_comp, comp_bytes));
-  const size_t reach_bytes = (size_t)ns * (2 * n / ts) * (2 * n / ts) * sizeof(float2);
+  const size_t reach_n = lazy ? (size_t)ns * (2 * n / ts) * (2 * n / ts) : 0;
+  const size_t reach_bytes = reach_n * sizeof(float2);
   RIX_TRY(ensure<R>(job, pt.ms_state, reach_bytes + 2 * (size_t)nblk * sizeof(Slot<R>) + 64));
   pt.ms_ncomp_cap = cap;
   RIX_CUDA(cudaMemsetAsync(pt.delta.p, 0, npix * sizeof(R), st));
@@ -1077,12 +1164,10 @@ int op_msclean(Job* job, int p, const rix_msclean_params* prm, R* delta_out, cud
   RIX_CUDA(cudaMemsetAsync(pt.sync.p, 0, sizeof(unsigned int), st));
   ca.barrier = pt.sync.as<unsigned int>();
   ca.status = job->status.as<int>();
-  {
-    const int64_t warps = (int64_t)ns * (2 * n / ts) * (2 * n / ts);
-    const int blocks = (int)std::min<int64_t>(ceil_div(warps, 8), (int64_t)ctx->num_sms * 8);
+  if (lazy) {
+    const int blocks = (int)std::min<int64_t>(ceil_div((int64_t)reach_n, 8), (int64_t)ctx->num_sms * 8);
     ::rix::note_launch();
-    if (ts == 32) k_clean_reach<R, 32><<<blocks, 256, 0, st>>>(ca, rch);
-    else k_clean_reach<R, 16><<<blocks, 256, 0, st>>>(ca, rch);
+    k_clean_reach<R><<<blocks, 256, 0, st>>>(ca, rch);
     RIX_LAUNCH_CHECK();
   }
   void* args[] = {&ca};
