@@ -291,14 +291,47 @@ struct TileArgs {
   int64_t ent_begin, ent_count;   // the partition's entries
   int64_t max_tile;         // ... of its fullest uv tile
   int* status;              // the job's status word (RIX_EINTERNAL on a failed check)
-  int slice, nsub;          // a work item is cut into nsub slices of `slice` entries (set_slices)
+  int slice, lsub;          // a work item is cut into 2^lsub slices of `slice` entries (set_slices)
 };
 
-// `sums`: the launch adds into the grid in FP32 (slice_entries)
+// The slices of a launch on `slots` CTAs (`sums`: it adds into the grid in FP32).
 void set_slices(TileArgs& a, int64_t slots, bool sums) {
   a.slice = slice_entries(a.ent_count, slots, sums ? a.max_tile : 0);
-  a.nsub = kItemEntries / a.slice;
+  a.lsub = slices_log2(a.max_tile, a.slice);
 }
+
+// A CTA's way through the slices: it looks 256 of them over at once and works
+// through those that hold entries.  One slice after the other, and on an even number
+// of CTAs, the dirty image of 500,001 coplanar samples at 1024^2, 30 to a tile, took
+// 593 instead of 181 us, in FP64 5.96 instead of 1.59 ms.
+struct SliceWalk {
+  uint2 list[256];   // entries [x, y) of the non-empty slices
+  int count[8];
+  // fills the list from slices first, first + gridDim, ... (in order); returns its
+  // length.  256 threads.
+  __device__ __forceinline__ int look(const TileArgs& a, int64_t first) {
+    const int64_t it = first + (int64_t)threadIdx.x * gridDim.x;
+    uint2 e = make_uint2(0u, 0u);
+    if (it < (a.item_count << a.lsub)) {
+      const int64_t item = a.item_begin + (it >> a.lsub);
+      e.x = a.items[item] + ((uint32_t)it & ((1u << a.lsub) - 1u)) * (uint32_t)a.slice;
+      e.y = min(a.items[item + 1], e.x + (uint32_t)a.slice);
+    }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned b = __ballot_sync(0xffffffffu, e.x < e.y);
+    if (lane == 0) count[warp] = __popc(b);
+    __syncthreads();
+    int before = __popc(b & ((1u << lane) - 1u)), n = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+      if (w < warp) before += count[w];
+      n += count[w];
+    }
+    if (e.x < e.y) list[before] = e;
+    __syncthreads();
+    return n;
+  }
+};
 
 // On the PSF's 2N grid (x_psf = 2 x exactly), an image-grid tile of side T
 // at tx T maps to first taps in [2 tx T + 3, 2 tx T + 2 T + 2]: the staged
@@ -388,11 +421,10 @@ __global__ void __launch_bounds__(256) k_tiles(TileArgs a) {
 
   // entries a warp takes at a time: all eight warps share a short slice
   const int wb = min(32, a.slice / nwarps);
-  for (int64_t it = blockIdx.x; it < a.item_count * a.nsub; it += gridDim.x) {
-    const int64_t item = a.item_begin + it / a.nsub;
-    const uint32_t e0 = a.items[item] + (uint32_t)((it % a.nsub) * a.slice);
-    const uint32_t e1 = min(a.items[item + 1], e0 + (uint32_t)a.slice);
-    if (e0 >= e1) continue;
+  __shared__ SliceWalk walk;
+  for (int64_t first = blockIdx.x; first < (a.item_count << a.lsub); first += 256 * (int64_t)gridDim.x)
+  for (int q = 0, nq = walk.look(a, first); q < nq; ++q) {
+    const uint32_t e0 = walk.list[q].x, e1 = walk.list[q].y;
     const uint32_t key = a.keys[e0];
     const int tx = (int)(key & tmask), ty = (int)((key >> a.bt) & tmask);
     const int p0 = (WW > 1) ? (int)((key >> (2 * a.bt)) & ((1u << a.bw) - 1u)) : 0;
@@ -555,7 +587,7 @@ int launch_tiles_impl(const Ctx* ctx, TileArgs a, cudaStream_t st) {
   per_sm = std::max(per_sm, 1);
   const int64_t slots = (int64_t)ctx->num_sms * per_sm;
   set_slices(a, slots, kUseGrid && sizeof(R) == 4);
-  const int64_t blocks = std::min<int64_t>(a.item_count * a.nsub, slots);
+  const int64_t blocks = slice_blocks(a.item_count << a.lsub, slots);
   if (blocks <= 0) return RIX_OK;
   timing_mark(kTimeTiles, st, true);
   ::rix::note_launch(); kern<<<(unsigned)blocks, 256, sm, st>>>(a);
@@ -619,11 +651,10 @@ __global__ void __launch_bounds__(256) k_tiles_ws(TileArgs a) {
   static_assert(kWsBatch % 8 == 0, "eight warps");
   constexpr int per_warp = kWsBatch / 8;
 
-  for (int64_t it = blockIdx.x; it < a.item_count * a.nsub; it += gridDim.x) {
-    const int64_t item = a.item_begin + it / a.nsub;
-    const uint32_t e0 = a.items[item] + (uint32_t)((it % a.nsub) * a.slice);
-    const uint32_t e1 = min(a.items[item + 1], e0 + (uint32_t)a.slice);
-    if (e0 >= e1) continue;
+  __shared__ SliceWalk walk;
+  for (int64_t first = blockIdx.x; first < (a.item_count << a.lsub); first += 256 * (int64_t)gridDim.x)
+  for (int q = 0, nq = walk.look(a, first); q < nq; ++q) {
+    const uint32_t e0 = walk.list[q].x, e1 = walk.list[q].y;
     const uint32_t key = a.keys[e0];
     const int tx = (int)(key & tmask), ty = (int)((key >> a.bt) & tmask);
     const int p0 = (int)((key >> (2 * a.bt)) & ((1u << a.bw) - 1u));
@@ -784,7 +815,7 @@ int launch_tiles_ws(const Ctx* ctx, TileArgs a, cudaStream_t st) {
   per_sm = std::max(per_sm, 1);
   const int64_t slots = (int64_t)ctx->num_sms * per_sm;
   set_slices(a, slots, sizeof(R) == 4);
-  const int64_t blocks = std::min<int64_t>(a.item_count * a.nsub, slots);
+  const int64_t blocks = slice_blocks(a.item_count << a.lsub, slots);
   if (blocks <= 0) return RIX_OK;
   timing_mark(kTimeTiles, st, true);
   ::rix::note_launch(); kern<<<(unsigned)blocks, 256, sm, st>>>(a);
