@@ -728,7 +728,16 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 && LOGL <= 12 ? 2 
 // in an instance of its own (CTAS = 0: the launch's size; with it in every launch
 // the phases' loops are loops again, 7.50 -> 7.57 ms for the 128 x 128 job).
 constexpr int kClusterCtas = 16;
-constexpr int kClusterLogL = 8;   // longest transform 2N that takes this path
+// The longest transform 2N that takes this path.  FP32 only: FP64 arithmetic keeps
+// 16 SMs busy long before the barrier counts (128 x 128, 30 iterations with Db4,
+// one and four levels, on the grid / a cluster: 3.18 / 4.07 and 4.58 / 5.44 ms; 64 x
+// 64 within 5 % either way).  With the concatenated dictionary, whose phases have
+// eight times the units, up to 64 x 64 (128 x 128, one and four levels: 1.71 / 2.44
+// and 2.59 / 3.05 ms).
+template <typename R, int DICT>
+constexpr int cluster_logl() {
+  return sizeof(R) == 8 ? 0 : DICT == RIX_DICT_DB4 ? 8 : 7;
+}
 
 template <typename R, int LOGL, int DICT, int CTAS>
 __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 2 : 1)
@@ -962,7 +971,7 @@ int launch_fista_loop(const Ctx* ctx, const FistaLoop<R>* f, int nb, cudaStream_
     }
   }
   args.t_tab = mom_host<R>(std::min(f[0].iters, kMomTab), args.mom_tab);
-  if constexpr (LOGL <= kClusterLogL) {
+  if constexpr (LOGL <= cluster_logl<R, DICT>()) {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
