@@ -1,8 +1,7 @@
 // FFT passes with the transform length, the batch and the radix plan fixed at
 // compile time, for the persistent minor-cycle loop.  Same Stockham
-// (autosort) ping-pong scheme, shared-memory padding and FP64-accurate
-// twiddle table as the run-time passes of fft_device.cuh; with every size a
-// constant, the 16 operand addresses of a radix item are one base register
+// (autosort) scheme, shared-memory padding and FP64-accurate twiddle table as the
+// row and column passes of fft_engine.cuh; with every size a constant, the 16 operand addresses of a radix item are one base register
 // plus immediate offsets and the item loops unroll.
 #pragma once
 
@@ -12,20 +11,20 @@ namespace rix {
 namespace {
 
 // radix (log2) of pass `ps` of a length-2^LOGL transform split into
-// ceil(LOGL / 4) passes of radix <= 16, the larger radices first
-__host__ __device__ constexpr int ct_npass(int logl) { return (logl + 3) / 4; }
-__host__ __device__ constexpr int ct_lr(int logl, int ps) {
+// ceil(LOGL / MLR) passes of radix <= 2^MLR, the larger radices first
+__host__ __device__ constexpr int ct_npass(int logl, int mlr = 4) { return (logl + mlr - 1) / mlr; }
+__host__ __device__ constexpr int ct_lr(int logl, int ps, int mlr = 4) {
   int logp = 0, lr = 0;
   for (int q = 0; q <= ps; ++q) {
-    const int rem = logl - logp, left = ct_npass(logl) - q;
+    const int rem = logl - logp, left = ct_npass(logl, mlr) - q;
     lr = (rem + left - 1) / left;
     logp += lr;
   }
   return lr;
 }
-__host__ __device__ constexpr int ct_logp(int logl, int ps) {
+__host__ __device__ constexpr int ct_logp(int logl, int ps, int mlr = 4) {
   int logp = 0;
-  for (int q = 0; q < ps; ++q) logp += ct_lr(logl, q);
+  for (int q = 0; q < ps; ++q) logp += ct_lr(logl, q, mlr);
   return logp;
 }
 

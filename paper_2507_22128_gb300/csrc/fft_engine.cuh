@@ -11,7 +11,8 @@
 // n the centred offset -M/2 .. M/2 - 1 (held at n mod M).  M = L is the single
 // transform e = 0.
 //
-// A thread carries 16 values in registers through every pass: global memory
+// A thread carries V = 16 values (fewer in FP64 at short lengths) in registers
+// through every pass: global memory
 // -> registers -> first pass, one shared-memory exchange between passes, last
 // pass -> registers -> global memory.
 //
@@ -58,10 +59,19 @@ struct XArgs {
   int pg;               // inverse rows: planes per grid row y
 };
 
+// Transforms of up to 2^kFewLogF points take fewer values per thread in FP64 (4, from
+// 2^8 on 8): the double-precision pipe takes a warp's instruction in 16 cycles or
+// more, so the 1,200 instructions of a thread with 16 values were 10 us of every pass
+// over a small image, however few its rows.  ms-CLEAN cycle of 20 components, four
+// partitions, 16 values / fewer: 32^2 3.1 / 1.6 ms, 128^2 3.8 / 1.8, 256^2 4.2 / 3.0,
+// 512^2 6.7 / 6.2.
+constexpr int kFewLogF = 9;
+
 // One transform length F = 2^LOGF, E = L / F sub-transforms; rows, or columns
 // with the thread index running over the CTA's columns first.
 //   T       F / 4 threads between 64 (short lengths: more CTAs for small
-//           images) and 256 (512 above 4096), 16 values each
+//           images) and 256 (512 above 4096), 16 values each; 128 threads
+//           with V = 4 or 8
 //   kCtas   CTAs per SM that the registers (WARPS in all) and the shared
 //           memory are sized for; one in FP64, whose rate of 1/64 of FP32
 //           leaves nothing for more warps to hide
@@ -69,11 +79,12 @@ struct XArgs {
 template <typename R, int LOGF, int E, bool COLS, int WARPS = 24>
 struct Xf {
   static constexpr int F = 1 << LOGF;
-  static constexpr int V = 16;
   static constexpr bool kF32 = sizeof(R) == 4;
+  static constexpr int V = kF32 || LOGF > kFewLogF ? 16 : LOGF < 8 ? 4 : 8;
+  static constexpr int MLR = V == 16 ? 4 : V == 8 ? 3 : 2;   // log2 of the largest radix
   static constexpr int kMaxT = F > 4096 ? 512 : 256;
   static constexpr int kWant = F / 4 < 64 ? 64 : F / 4;
-  static constexpr int T = kWant < kMaxT ? kWant : kMaxT;
+  static constexpr int T = V < 16 ? 128 : kWant < kMaxT ? kWant : kMaxT;
   static constexpr int NB = T * V / F;                 // rows (columns) per CTA
   static constexpr int PADF = padded_len(F);
   static constexpr int kBuf = NB * PADF;               // complex values of an exchange buffer
@@ -82,10 +93,10 @@ struct Xf {
   static constexpr size_t kStash = (size_t)(E == 2 ? T * V : 0) * 2 * sizeof(R);
   static constexpr bool kPing = kF32 && kCtas * (2 * kBuf * 2 * sizeof(R) + kStash) <= 220 * 1024;
   static constexpr size_t kSmem = (size_t)(kPing ? 2 : 1) * kBuf * 2 * sizeof(R) + kStash;
-  static constexpr int NP = ct_npass(LOGF);
-  static constexpr int LRL = ct_lr(LOGF, NP - 1);      // radix of the last pass
+  static constexpr int NP = ct_npass(LOGF, MLR);
+  static constexpr int LRL = ct_lr(LOGF, NP - 1, MLR); // radix of the last pass
   static constexpr int IPRL = F >> LRL;
-  static constexpr int LR0 = ct_lr(LOGF, 0);
+  static constexpr int LR0 = ct_lr(LOGF, 0, MLR);
   static constexpr int IPR0 = F >> LR0;
   // item `it` of the thread in a pass with 2^LR legs: row (column) c and the
   // position i of leg 0; leg r sits at i + r IPR.  Slot s = it 2^LR + r.
@@ -128,11 +139,11 @@ __host__ __device__ constexpr int fold(int r) {
 // next exchange (ping-pong); without ping-pong every exchange waits until the
 // buffer has been read.
 template <class X, typename R, int DIR, int LOGF, int PS, bool kPad = false>
-__device__ __forceinline__ void xf_passes(cplx<R> (&v)[16], cplx<R>* buf, int& par, const cplx<R>* __restrict__ tw,
+__device__ __forceinline__ void xf_passes(cplx<R> (&v)[X::V], cplx<R>* buf, int& par, const cplx<R>* __restrict__ tw,
                                           int tid) {
   using C = cplx<R>;
-  constexpr int LR = ct_lr(LOGF, PS), LOGP = ct_logp(LOGF, PS);
-  constexpr int RAD = 1 << LR, IPR = X::F >> LR, P = 1 << LOGP, K = 16 / RAD;
+  constexpr int LR = ct_lr(LOGF, PS, X::MLR), LOGP = ct_logp(LOGF, PS, X::MLR);
+  constexpr int RAD = 1 << LR, IPR = X::F >> LR, P = 1 << LOGP, K = X::V / RAD;
 #pragma unroll
   for (int it = 0; it < K; ++it) {
     C* w = v + it * RAD;
@@ -157,8 +168,8 @@ __device__ __forceinline__ void xf_passes(cplx<R> (&v)[16], cplx<R>* buf, int& p
     else dft<RAD, DIR>(w);
   }
   if constexpr (PS + 1 < X::NP) {
-    constexpr int LRN = ct_lr(LOGF, PS + 1);
-    constexpr int RADN = 1 << LRN, IPRN = X::F >> LRN, KN = 16 / RADN, PST = X::kPosStride;
+    constexpr int LRN = ct_lr(LOGF, PS + 1, X::MLR);
+    constexpr int RADN = 1 << LRN, IPRN = X::F >> LRN, KN = X::V / RADN, PST = X::kPosStride;
     // padi is linear over multiples of 16 and inside one group of 16
     constexpr bool kLin16 = (P % 16) == 0;
     constexpr bool kLinSmall = (P * RAD <= 16) && (16 % (P * RAD) == 0);
@@ -208,14 +219,14 @@ __device__ __forceinline__ int opaque_tid() {
 // slots, T apart) e = 1's; on return v holds the last one's outputs and
 // stash, with E = 2, the first one's.
 template <class X, typename R, int DIR, int LOGF, int E>
-__device__ __forceinline__ void xf_run(cplx<R> (&v)[16], cplx<R>* buf, cplx<R>* stash, int& par,
+__device__ __forceinline__ void xf_run(cplx<R> (&v)[X::V], cplx<R>* buf, cplx<R>* stash, int& par,
                                        const cplx<R>* __restrict__ tw) {
 #pragma unroll 1
   for (int e = 0;; ++e) {
     xf_passes<X, R, DIR, LOGF, 0>(v, buf, par, tw, opaque_tid());
     if (e == E - 1) break;
 #pragma unroll
-    for (int s = 0; s < 16; ++s) {
+    for (int s = 0; s < X::V; ++s) {
       const cplx<R> t = stash[s * X::T];
       stash[s * X::T] = v[s];
       v[s] = t;
@@ -280,9 +291,9 @@ __global__ void __launch_bounds__((Xf<R, LOGF, E, false>::T), (Xf<R, LOGF, E, fa
   const R* corr = static_cast<const R*>(a.corr);
   const C* scr = a.mode == kFacPhase && a.screen ? static_cast<const C*>(a.screen) + (int64_t)p * M * M : nullptr;
   const double wp = a.w0 + p * a.dw;
-  C v[16];
+  C v[X::V];
 #pragma unroll
-  for (int s = 0; s < 16; ++s) {
+  for (int s = 0; s < X::V; ++s) {
     int c, n;
     X::template slot<X::LR0>(tid, s, c, n);
     const int aa = (n + M / 2) & (M - 1), b = b0 + c;
@@ -299,7 +310,7 @@ __global__ void __launch_bounds__((Xf<R, LOGF, E, false>::T), (Xf<R, LOGF, E, fa
   }
   if constexpr (E == 2) {
 #pragma unroll
-    for (int s = 0; s < 16; ++s) {
+    for (int s = 0; s < X::V; ++s) {
       int c, n;
       X::template slot<X::LR0>(tid, s, c, n);
       stash[s * X::T] = cmul(v[s], half_twiddle<R, LOGF, -1>(tw, n));
@@ -308,7 +319,7 @@ __global__ void __launch_bounds__((Xf<R, LOGF, E, false>::T), (Xf<R, LOGF, E, fa
   xf_run<X, R, -1, LOGF, E>(v, buf, stash, par, tw);
   C* Tp = T + (int64_t)p * t_plane(a.S, M);
 #pragma unroll
-  for (int s = 0; s < 16; ++s) {
+  for (int s = 0; s < X::V; ++s) {
     int c, k;
     X::template slot<X::LRL>(tid, s, c, k);
     const int b = b0 + c, j = E * k - a.lo;
@@ -475,9 +486,9 @@ __global__ void __launch_bounds__((Xf<R, LOGF, E, true>::T), (Xf<R, LOGF, E, tru
   RIX_X_SMEM
   const int p = blockIdx.y, j0 = blockIdx.x * X::NB;
   const C* Tp = T + (int64_t)p * t_plane(a.S, M);
-  C v[16];
+  C v[X::V];
 #pragma unroll
-  for (int s = 0; s < 16; ++s) {
+  for (int s = 0; s < X::V; ++s) {
     int c, n;
     X::template slot<X::LR0>(tid, s, c, n);
     const int j = j0 + c;
@@ -485,7 +496,7 @@ __global__ void __launch_bounds__((Xf<R, LOGF, E, true>::T), (Xf<R, LOGF, E, tru
   }
   if constexpr (E == 2) {
 #pragma unroll
-    for (int s = 0; s < 16; ++s) {
+    for (int s = 0; s < X::V; ++s) {
       int c, n;
       X::template slot<X::LR0>(tid, s, c, n);
       stash[s * X::T] = cmul(v[s], half_twiddle<R, LOGF, -1>(tw, n));
@@ -495,7 +506,7 @@ __global__ void __launch_bounds__((Xf<R, LOGF, E, true>::T), (Xf<R, LOGF, E, tru
   C* sp = spec + (int64_t)p * a.S * a.S;
   const bool even = ((a.lo | a.S) & 1) == 0;
 #pragma unroll
-  for (int s = 0; s < 16; ++s) {
+  for (int s = 0; s < X::V; ++s) {
     int c, k;
     X::template slot<X::LRL>(tid, s, c, k);
     const int j = j0 + c, i = E * k - a.lo;
@@ -528,9 +539,9 @@ __global__ void __launch_bounds__((Xf<R, LOGF, E, true>::T), (Xf<R, LOGF, E, tru
   const C* sp = spec + (int64_t)p * a.S * a.S;
   const C zero = cmake<C>(0.0, 0.0);
   const bool even = ((a.lo | a.S) & 1) == 0;
-  C v[16];
+  C v[X::V];
 #pragma unroll
-  for (int s = 0; s < 16; ++s) {
+  for (int s = 0; s < X::V; ++s) {
     int c, k;
     X::template slot<X::LR0>(tid, s, c, k);
     const int j = j0 + c, i = E * k - a.lo;
@@ -558,7 +569,7 @@ __global__ void __launch_bounds__((Xf<R, LOGF, E, true>::T), (Xf<R, LOGF, E, tru
   xf_run<X, R, +1, LOGF, E>(v, buf, stash, par, tw);
   C* Tp = T + (int64_t)p * t_plane(a.S, M);
 #pragma unroll
-  for (int s = 0; s < 16; ++s) {
+  for (int s = 0; s < X::V; ++s) {
     int c, n;
     X::template slot<X::LRL>(tid, s, c, n);
     const int j = j0 + c;
@@ -580,9 +591,9 @@ __global__ void __launch_bounds__((Xf<R, LOGF, 2, true>::T), (Xf<R, LOGF, 2, tru
   constexpr int M = X::F, L = 2 * M;
   RIX_X_SMEM
   const int j0 = blockIdx.x * X::NB;
-  C v[16];
+  C v[X::V];
 #pragma unroll
-  for (int s = 0; s < 16; ++s) {
+  for (int s = 0; s < X::V; ++s) {
     int c, n;
     X::template slot<X::LR0>(tid, s, c, n);
     const int j = j0 + c;
@@ -599,7 +610,7 @@ __global__ void __launch_bounds__((Xf<R, LOGF, 2, true>::T), (Xf<R, LOGF, 2, tru
     if constexpr (X::kPing) par ^= 1;
     else __syncthreads();
 #pragma unroll
-    for (int s = 0; s < 16; ++s) {
+    for (int s = 0; s < X::V; ++s) {
       int c, k;
       X::template slot<X::LRL>(tid, s, c, k);
       const int j = j0 + c;
@@ -609,7 +620,7 @@ __global__ void __launch_bounds__((Xf<R, LOGF, 2, true>::T), (Xf<R, LOGF, 2, tru
     }
     __syncthreads();
 #pragma unroll
-    for (int s = 0; s < 16; ++s) {
+    for (int s = 0; s < X::V; ++s) {
       int c, k;
       X::template slot<X::LR0>(tid, s, c, k);
       v[s] = b[X::addr(c, k)];
@@ -619,14 +630,14 @@ __global__ void __launch_bounds__((Xf<R, LOGF, 2, true>::T), (Xf<R, LOGF, 2, tru
     // the first pass's own slots hold e = 1's input; the last pass's results
     // of e = 0 take their place slot by slot
 #pragma unroll
-    for (int s = 0; s < 16; ++s) {
+    for (int s = 0; s < X::V; ++s) {
       const C t = stash[s * X::T];
       stash[s * X::T] = v[s];
       v[s] = t;
     }
   }
 #pragma unroll
-  for (int s = 0; s < 16; ++s) {
+  for (int s = 0; s < X::V; ++s) {
     int c, n;
     X::template slot<X::LRL>(tid, s, c, n);
     const int j = j0 + c;
@@ -652,16 +663,16 @@ __global__ void __launch_bounds__((Xf<R, LOGF, E, false>::T), (Xf<R, LOGF, E, fa
   img += (int64_t)blockIdx.y * M * M;
   const R* corr = static_cast<const R*>(a.corr);
   const C zero = cmake<C>(0.0, 0.0);
-  R acc[16];
+  R acc[X::V];
 #pragma unroll
-  for (int s = 0; s < 16; ++s) acc[s] = R(0);
+  for (int s = 0; s < X::V; ++s) acc[s] = R(0);
 #pragma unroll 1
   for (int p = pb; p < pe; ++p) {
     tid = opaque_tid();
     const C* Tp = T + (int64_t)p * t_plane(a.S, M);
-    C v[16];
+    C v[X::V];
 #pragma unroll
-    for (int s = 0; s < 16; ++s) {
+    for (int s = 0; s < X::V; ++s) {
       int c, k;
       X::template slot<X::LR0>(tid, s, c, k);
       const int b = b0 + c, j = E * k - a.lo;
@@ -691,7 +702,7 @@ __global__ void __launch_bounds__((Xf<R, LOGF, E, false>::T), (Xf<R, LOGF, E, fa
     xf_run<X, R, +1, LOGF, E>(v, buf, stash, par, tw);
     const double wp = a.w0 + p * a.dw;
 #pragma unroll
-    for (int s = 0; s < 16; ++s) {
+    for (int s = 0; s < X::V; ++s) {
       int c, n;
       X::template slot<X::LRL>(tid, s, c, n);
       const int64_t pix = (int64_t)(b0 + c) * M + ((n + M / 2) & (M - 1));
@@ -710,7 +721,7 @@ __global__ void __launch_bounds__((Xf<R, LOGF, E, false>::T), (Xf<R, LOGF, E, fa
     }
   }
 #pragma unroll
-  for (int s = 0; s < 16; ++s) {
+  for (int s = 0; s < X::V; ++s) {
     int c, n;
     X::template slot<X::LRL>(tid, s, c, n);
     const int b = b0 + c, aa = (n + M / 2) & (M - 1);
