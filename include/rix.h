@@ -297,9 +297,10 @@ int rix_minor_cycle_fista(rix_job_t job, int part, const rix_fista_params* param
  * the loops of the batch run as a dataflow (each phase of a loop waits only
  * for the previous phase of the same loop, so one loop's phase ends are
  * filled with the others' work); with the concatenated dictionary they
- * advance together, one grid barrier per phase serving all of them; on images
- * up to 128^2 each loop runs on a thread-block cluster of its own.  Every
- * device-side poll is bounded (RIX_ETIMEOUT at rix_job_sync). */
+ * advance together, one grid barrier per phase serving all of them; on FP32
+ * images up to 128^2 (64^2 with the concatenated dictionary) each loop runs on a
+ * thread-block cluster of its own.  Every device-side poll is bounded
+ * (RIX_ETIMEOUT at rix_job_sync). */
 int rix_minor_cycle_fista_batch(rix_job_t job, int n_parts, const int32_t* parts, const rix_fista_params* params,
                                 rix_stream_t stream);
 

@@ -145,10 +145,12 @@ __device__ __forceinline__ cplx<R> wscreen(double wp, double nm1) {
 }
 
 // exp(DIR 2 pi i w (n-1)) in FP32 with w = wh + wl and n - 1 = m.x + m.y held as
-// pairs of floats (48 bits): the product's leading part is reduced exactly and
-// the rest added, so the turn is as accurate as FP64's after its rounding to
-// float (the leading product is below 2^23 turns, its remainders below 1e-6),
-// at eight FP32 operations instead of five FP64 ones at 1/64 of their rate
+// pairs of floats (48 bits): the leading product is reduced to a fraction of a turn
+// exactly; what it lost to rounding (up to 2^-24 of its turns) and the two cross
+// products are added in FP32.  Left out are 2^-24 of those additions and wl m.y,
+// 2^-48 of the turns: below the rounding of the result to float up to some
+// thousand turns.  Eight FP32 operations instead of five FP64 ones at 1/64 of
+// their rate
 template <int DIR>
 __device__ __forceinline__ float2 wscreen_ff(float wh, float wl, float2 m) {
   const float p = __fmul_rn(wh, m.x);

@@ -1,17 +1,17 @@
 // a4-a7: G^dagger F and F^dagger G of Eq. 2 for one uv partition.
 //
 // Model image -> w-planes (correction, phase screen, pruned FFT; k_fft.cu)
-// -> per work item (one uv tile of one w-plane block, at most 2048 sorted
-// samples): stage the tile (+ kernel halo) of the 8 model planes it touches
-// into shared memory, degrid each sample with a warp (32 lanes x 16 taps,
-// warp-shuffle reduction), form the weighted residual, spread it into a
-// shared-memory sub-grid, and flush that sub-grid once per work item with
-// vector atomics -> residual planes -> inverse pruned FFT, conjugate phase
-// screen, sum over planes, correction -> residual image.
+// -> per slice of a work item (one uv tile of one w-plane block, at most 2048
+// sorted samples): stage the tile (+ kernel halo) of the model planes it touches
+// into shared memory, degrid each sample with a group of lanes (warp-shuffle
+// reduction), form the weighted residual, spread it into a shared-memory sub-grid,
+// and add that sub-grid once per slice with vector atomics -> residual planes ->
+// inverse pruned FFT, conjugate phase screen, sum over planes, correction ->
+// residual image.  FP32 w-stacked jobs take k_tiles_fp.cu between the transforms.
 //
-// Precision: sample coordinates, the kernel argument offsets and the w-plane
-// phases are formed in FP64; kernel weights, accumulation and FFTs in the
-// job's precision (FP32 or FP64).
+// Precision: sample coordinates and the kernel argument offsets are formed in
+// FP64, the w-plane phases in FP64 or, for FP32 PSFs, from pairs of floats;
+// kernel weights, accumulation and FFTs in the job's precision (FP32 or FP64).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -596,8 +596,8 @@ int launch_tiles_impl(const Ctx* ctx, TileArgs a, cudaStream_t st) {
   return RIX_OK;
 }
 
-// ---- w-stacked gridding without shared-memory atomics ----------------------
-// Phase A: each warp degrids 4 samples of a 32-sample batch (32 lanes x 16
+// ---- FP64 w-stacked gridding without shared-memory atomics -----------------
+// (FP32 jobs: k_tiles_fp.cu.)  Phase A: each warp degrids 4 samples of a 32-sample batch (32 lanes x 16
 // taps, shuffle reduction) and stores per-sample records (weighted residual,
 // tap origin, the 24 kernel weights).  Phase B: warp w owns w-plane w of the
 // staged sub-grid and applies every record of the batch to it with plain
@@ -610,29 +610,21 @@ template <int T, int MODE> struct WsGeom {
   static constexpr int PL = ((SP * SPP + 7) / 16) * 16 + 8;                // plane stride, 8 mod 16
 };
 
-template <typename R>
-struct alignas(4 * sizeof(R)) WsRecord {
-  // header, one vector load: weighted residual and the tap origin (ou | ov << 8)
-  R yr, yi;
-  uint32_t ouv;
-  uint32_t pad[sizeof(R) == 8 ? 3 : 1];   // the weights start on a 4 sizeof(R) boundary
+struct alignas(32) WsRecord {
+  double yr, yi;                          // weighted residual, one 16-byte load
+  uint32_t ouv;                           // the tap origin (ou | ov << 8)
+  uint32_t pad[3];
   // u weights in pairs (u_i, u_{i+4}) at [2i, 2i + 1] for i < 4, then the 8
   // v weights and the 8 w weights
-  R w[3 * kW];
+  double w[3 * kW];
 };
-
-// header of a record as loaded by phase B
-static_assert(offsetof(WsRecord<double>, w) == 32 && sizeof(WsRecord<double>) % 32 == 0, "record layout");
-template <typename R> struct WsHead { R yr, yi; uint32_t ouv; };
-__device__ __forceinline__ WsHead<double> ws_head(const WsRecord<double>& r) {
-  const double2 h = *reinterpret_cast<const double2*>(&r);
-  return {h.x, h.y, r.ouv};
-}
+static_assert(offsetof(WsRecord, w) == 32 && sizeof(WsRecord) % 32 == 0, "record layout");
 
 constexpr int kWsBatch = 32;
 
-template <typename R, int T, int MODE>
+template <int T, int MODE>
 __global__ void __launch_bounds__(256) k_tiles_ws(TileArgs a) {
+  using R = double;
   using C = cplx<R>;
   using TG = WsGeom<T, MODE>;
   constexpr int SP = TG::SP, SPP = TG::SPP, PL = TG::PL;
@@ -640,7 +632,7 @@ __global__ void __launch_bounds__(256) k_tiles_ws(TileArgs a) {
   extern __shared__ __align__(32) unsigned char smem_raw[];
   C* sm_model = reinterpret_cast<C*>(smem_raw);
   C* sm_grid = sm_model + (kUseModel ? kW * PL : 0);
-  WsRecord<R>* rec = reinterpret_cast<WsRecord<R>*>(sm_grid + kW * PL);
+  WsRecord* rec = reinterpret_cast<WsRecord*>(sm_grid + kW * PL);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
   const int64_t SS = (int64_t)a.S * a.S;
@@ -720,7 +712,7 @@ __global__ void __launch_bounds__(256) k_tiles_ws(TileArgs a) {
             accr[q] = acci[q] = R(0);
             if constexpr (kUseModel) {
               const int kou = __shfl_sync(0xffffffffu, ou, j + q), kov = __shfl_sync(0xffffffffu, ov, j + q);
-              const WsRecord<R>& rc = rec[j0 + j + q];
+              const WsRecord& rc = rec[j0 + j + q];
               const int vrow = lane & 7, plh = lane >> 3;
               const R wv = rc.w[kW + vrow];
 #pragma unroll
@@ -753,7 +745,7 @@ __global__ void __launch_bounds__(256) k_tiles_ws(TileArgs a) {
           // lane j + q holds its entry's data; lanes past nb wrote no record
           const int q = lane - j;
           if (q >= 0 && q < 2 && j0 + lane < nb) {
-            WsRecord<R>& rc = rec[j0 + lane];
+            WsRecord& rc = rec[j0 + lane];
             rc.yr = wt * (vre - (q ? accr[1] : accr[0]));
             rc.yi = wt * (vim - (q ? acci[1] : acci[0]));
             rc.ouv = (uint32_t)ou | ((uint32_t)ov << 8);
@@ -766,13 +758,13 @@ __global__ void __launch_bounds__(256) k_tiles_ws(TileArgs a) {
         const int vrow = lane & 7, ig = lane >> 3;
         C* gpl = sm_grid + warp * PL;
         for (int k = 0; k < nb; ++k) {
-          const WsRecord<R>& rc = rec[k];
-          const WsHead<R> hd = ws_head(rc);
+          const WsRecord& rc = rec[k];
+          const double2 y = *reinterpret_cast<const double2*>(&rc.yr);
+          const uint32_t ouv = rc.ouv;
           const R f = rc.w[2 * kW + warp] * rc.w[kW + vrow];
-          const R cr = hd.yr * f, ci = hd.yi * f;
-          C* cell = gpl + ((int)(hd.ouv & 0xffu) + ig) * SPP + (int)(hd.ouv >> 8) + vrow;
-          using R2 = cplx<R>;
-          const R2 wp = *reinterpret_cast<const R2*>(&rc.w[2 * ig]);
+          const R cr = y.x * f, ci = y.y * f;
+          C* cell = gpl + ((int)(ouv & 0xffu) + ig) * SPP + (int)(ouv >> 8) + vrow;
+          const double2 wp = *reinterpret_cast<const double2*>(&rc.w[2 * ig]);
           const R w0 = wp.x, w1 = wp.y;
           C g0 = cell[0], g1 = cell[4 * SPP];
           g0.x += cr * w0; g0.y += ci * w0;
@@ -791,30 +783,26 @@ __global__ void __launch_bounds__(256) k_tiles_ws(TileArgs a) {
       const C val = sm_grid[pl * PL + iu * SPP + iv];
       if ((val.x != R(0) || val.y != R(0)) && u >= 0 && u < a.S && v >= 0 && v < a.S) {
         C* dst = &out[(p0 + pl) * SS + (int64_t)u * a.S + v];
-        if constexpr (sizeof(R) == 4) {
-          atomicAdd(reinterpret_cast<float2*>(dst), *reinterpret_cast<const float2*>(&val));
-        } else {
-          atomicAdd(&dst->x, val.x);
-          atomicAdd(&dst->y, val.y);
-        }
+        atomicAdd(&dst->x, val.x);
+        atomicAdd(&dst->y, val.y);
       }
     }
     __syncthreads();
   }
 }
 
-template <typename R, int T, int MODE>
+template <int T, int MODE>
 int launch_tiles_ws(const Ctx* ctx, TileArgs a, cudaStream_t st) {
   using TG = WsGeom<T, MODE>;
   constexpr bool kUseModel = (MODE == kResid);
-  const size_t sm = (size_t)(int(kUseModel) + 1) * kW * TG::PL * sizeof(cplx<R>) + kWsBatch * sizeof(WsRecord<R>);
-  auto kern = k_tiles_ws<R, T, MODE>;
+  const size_t sm = (size_t)(int(kUseModel) + 1) * kW * TG::PL * sizeof(double2) + kWsBatch * sizeof(WsRecord);
+  auto kern = k_tiles_ws<T, MODE>;
   RIX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   int per_sm = 0;
   RIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, sm));
   per_sm = std::max(per_sm, 1);
   const int64_t slots = (int64_t)ctx->num_sms * per_sm;
-  set_slices(a, slots, sizeof(R) == 4);
+  set_slices(a, slots, false);
   const int64_t blocks = slice_blocks(a.item_count << a.lsub, slots);
   if (blocks <= 0) return RIX_OK;
   timing_mark(kTimeTiles, st, true);
@@ -836,7 +824,7 @@ int launch_tiles(const Job* job, const TileArgs& a, cudaStream_t st) {
     } else if constexpr (MODE == kDegrid) {
       return launch_tiles_impl<R, kW, 16, MODE>(job->ctx, a, st);
     } else {
-      return launch_tiles_ws<R, 16, MODE>(job->ctx, a, st);
+      return launch_tiles_ws<16, MODE>(job->ctx, a, st);
     }
   }
   if (job->tile == 16) return launch_tiles_impl<R, 1, 16, MODE>(job->ctx, a, st);

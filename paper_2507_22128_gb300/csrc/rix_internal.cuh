@@ -344,8 +344,8 @@ struct Job {
   DevBuf keys, samples, items;              // entries and work-item begin offsets (+1 sentinel)
   // Gridder order: within every work item the entries are reordered by their
   // first tap (the cell their kernel footprint starts at), so runs of
-  // entries with one footprint are contiguous; a chunk is a run of at most 32
-  // such entries.  egeom and gsamples are in this order; `samples` keeps the
+  // entries with one footprint are contiguous; a chunk is a run of at most
+  // chunk_limit such entries.  egeom and gsamples are in this order; `samples` keeps the
   // sorted order rix_get_sorted_entries reports.
   DevBuf egeom;                             // per entry: kernel offsets and tap origin (EntryGeom<R>)
   DevBuf gsamples;                          // per entry: sample index
@@ -368,7 +368,7 @@ struct Job {
   // streams the job's calls ran on, each with an event recorded after the call
   std::vector<std::pair<cudaStream_t, cudaEvent_t>> touched;
   // tuning of the FP32 w-stacked gridder (rix_job_tune): entries per chunk
-  // (at most 32) and resident CTAs per SM (0: as many as fit)
+  // (at most 256) and resident CTAs per SM (0: as many as fit)
   int chunk_limit = 64;
   int fp_ctas_per_sm = 0;
   bool gorder = false;   // egeom (and gsamples) in the gridder order
